@@ -107,8 +107,9 @@ typedef struct {
 
 /* Kernel families with their own configurations: REDUCE (pr_reduce*),
  * SEGMENTED (pr_segmented_reduce*, and rows that do not fit ROWS), BACKWARD
- * (pr_reduce_backward), ROWS (pr_reduce_rows when cols is a whole number of
- * vectors and x is aligned to the vector width; bucketed by rows*cols), AXIS
+ * (pr_reduce_backward), ROWS (pr_reduce_rows for few long rows when cols is a
+ * whole number of vectors and x is aligned to the vector width; bucketed by
+ * rows*cols; shorter or more rows ignore it: groups of lanes take a row each), AXIS
  * (pr_reduce_axis with inner > 1; bucketed by outer*n*inner: block and
  * blocks_per_sm size the warps in flight, unroll the rows in flight per lane,
  * vec_bytes the column vectors when a row is a whole number of them). */

@@ -529,6 +529,65 @@ static pr_status run_rows(const void* x, int64_t rows, int64_t cols, int dtype, 
     return PR_OK;
 }
 
+// Lanes per row (log2) of k_rows_group for `rows` rows of `nv` 32-byte vectors
+// on `sms` SMs; -1: the rows are too few and too long for it, and k_rows or
+// k_segmented, which split the elements evenly over the SMs, take them.
+// Measured on GB300 (us; the group kernel against the kernel that had the shape):
+//   four vectors a lane: [200000, 120] fp32 sum 1 / 2 / 4 / 8 / 32 lanes 22.2 /
+//     18.2 / 18.2 / 20.6 / 55 (k_rows 968), [32768, 1000] with index 8 / 32
+//     lanes 26.7 / 26.7 (422);
+//   the whole block from 1024 vectors a row: [2048, 8192] 16.0 with a warp,
+//     13.4 with a block; 512 vectors ([8192, 4096]) 22.6 and 26.7 (47.3);
+//   fewer than 16 rows per SM leave warps idle, so from 256 vectors they take
+//     blocks too;
+//   the even split where a row per block loads the SMs unevenly: [64, 32768]
+//     fp32 7.7 and 7.7, [300, 65536] 16.4 (16.6), and sooner for 8-byte types,
+//     some of which are bound by arithmetic: fp64 minimum with index [500,
+//     16384] 25.5 (28.3), [300, 32768] 27.1 (25.4), [700, 32768] 62.5 (57.5).
+static int rows_group_lanes(int64_t rows, int64_t nv, int es, int sms) {
+    const bool wide = es == 8;
+    if (nv > ((int64_t)1 << 24) || (rows * 3 < (int64_t)sms * 5 && nv > 4096)) return -1;
+    if (rows < (int64_t)sms * (wide ? 8 : 4) && nv > (wide ? 4096 : 8192)) return -1;
+    if (nv >= 1024 || (nv >= 256 && rows < 16 * (int64_t)sms)) return 8;
+    int gl = 0;
+    while (gl < 5 && ((int64_t)4 << gl) < nv) gl++;
+    // few rows: more lanes each, down to one vector a lane
+    while (gl < 5 && ((int64_t)1 << gl) < nv && (rows << gl) < (int64_t)sms * 1024) gl++;
+    return gl;
+}
+
+// Rows by groups of lanes (any length and alignment); PR_ERR_UNSUPPORTED
+// (nothing enqueued, no message kept) when they are left to the other kernels.
+static pr_status run_rows_group(const void* x, int64_t rows, int64_t cols, int dtype, int op, int prec, int aux,
+                                void* out, int64_t* argidx, pr_prod_aux* paux, cudaStream_t st) {
+    const int es = elem_size(dtype);
+    const uintptr_t mis = reinterpret_cast<uintptr_t>(x) % kGroupVec;
+    if (rows < 1 || rows > (int64_t)1 << 50 || cols < 1 || mis % es) return PR_ERR_UNSUPPORTED;
+    const KernelEntry* e = reg_find(KernelKey{K_ROWS_GROUP, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux, 0, 0});
+    if (!e) return PR_ERR_UNSUPPORTED;
+    DevInfo di;
+    pr_status s = device_info(&di, nullptr);
+    if (s != PR_OK) return s;
+    // whole vectors, or one more where rows start off the vector grid
+    const int64_t ve = kGroupVec / es;
+    const int64_t nv = cols % ve == 0 && mis == 0 ? cols / ve : cols / ve + 2;
+    const int gl = rows_group_lanes(rows, nv, es, di.sms);
+    if (gl < 0) return PR_ERR_UNSUPPORTED;
+    const int64_t grid = ((rows << gl) + kGroupBlock - 1) / kGroupBlock;
+    if (grid > 0x7fffffff) return PR_ERR_UNSUPPORTED;
+    // (the kernel needs no workspace, but the stream gets its own as with
+    // every other kernel, so that what a first call on a stream does and
+    // refuses does not depend on the shape)
+    Workspace ws;
+    s = get_ws(st, &ws);
+    if (s != PR_OK) return s;
+    RowGroupArgs a{x, rows, cols, (int)mis / es, gl, out, argidx, paux};
+    PR_INJECT_LAUNCH();
+    cudaError_t err = reinterpret_cast<RowGroupLaunch>(e->launch)(a, (int)grid, kGroupBlock, st);
+    if (err != cudaSuccess) return fail(PR_ERR_CUDA, "row launch: %s", cudaGetErrorString(err));
+    return PR_OK;
+}
+
 constexpr int kBwdWaves = 8;  // backward grid = resident blocks x this (capped at the chunk count)
 
 static pr_status run_backward(int op, int dtype, const void* x, int64_t rows, int64_t cols, const void* g,
@@ -912,14 +971,17 @@ pr_status pr_reduce_rows(const void* x, int64_t rows, int64_t cols, pr_dtype dty
     if (rows < 0 || cols < 0) return fail(PR_ERR_INVALID, "rows and cols must be >= 0");
     if (cols > 0 && rows > ((int64_t)1 << 62) / cols) return fail(PR_ERR_INVALID, "rows*cols overflows");
     if (rows > 0 && cols > 0 && !x) return fail(PR_ERR_INVALID, "x is NULL");
-    // Rows whose length is a whole number of vectors, on an aligned x, take
-    // the row kernel; anything else the general segmented kernel.
+    // Rows by groups of lanes (rows_group_lanes); the few long rows it leaves
+    // take the row kernel where their length is a whole number of vectors and
+    // x is aligned, else the general segmented kernel.
     if (rows > 0 && cols > 0 && out && check_common(dtype, op, precision) == PR_OK &&
         !(argidx && op != PR_MAX && op != PR_MIN) && !(aux && !(op == PR_PROD && (dtype == PR_F32 || dtype == PR_F64)))) {
         ensure_registered();
         const int auxk = argidx ? AUX_ARG : (aux ? AUX_PROD : AUX_NONE);
+        pr_status s = run_rows_group(x, rows, cols, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream);
+        if (s != PR_ERR_UNSUPPORTED) return s;
         const pr_config c = lookup_cfg(PR_KIND_ROWS, dtype, op, precision, rows * cols);
-        const pr_status s = run_rows(x, rows, cols, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream, c);
+        s = run_rows(x, rows, cols, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream, c);
         if (s != PR_ERR_UNSUPPORTED) return s;
         g_msg.clear();
     }

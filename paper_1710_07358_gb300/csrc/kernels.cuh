@@ -51,6 +51,18 @@
 //   last of them to finish (per-row ticket) combines them in block order, so
 //   results are deterministic for a fixed launch configuration.
 //
+// k_rows_group  equal rows of any length and alignment, short ones above all:
+//   a row goes to a group of 2^gl neighbouring lanes of a warp (gl <= 5) or
+//   to a whole block, and ends with a combine across those lanes only.  k_rows
+//   and k_segmented end every row with a combine of the whole block, about
+//   1.2 us during which the block streams nothing: a row of a megabyte hides
+//   it, one of a few kilobytes does not.  Bound by HBM from a few kilobytes a
+//   row (fp32 sum of [32768, 1000] 174 -> 22.6 us, 0.86 of a 6.8 TB/s copy;
+//   [8192, 4096] 47 -> 22.6), by the latency of each row's short chain below
+//   ([200000, 120] 968 -> 18.2 us, 0.78; maximum with index of [32768, 1000]
+//   397 -> 26.7).  No grid loop: a block per 256 threads of work, so that the
+//   hardware evens out the rows.
+//
 // k_combine_parts  one block combining an array of partials in order.
 #pragma once
 #include <type_traits>
@@ -60,6 +72,8 @@ namespace pr {
 
 constexpr int kSlot = 64;      // bytes per partial slot (>= sizeof(Part) of every trait)
 constexpr int kSmallSeg = 512; // segments up to this length are reduced by one warp
+constexpr int kGroupBlock = 256;   // threads per block of the group kernels
+constexpr int kGroupVec = 32;      // bytes per vector load
 enum : int { kErrInvalid = 1, kErrTimeout = 4 };
 
 struct Workspace {
@@ -112,6 +126,16 @@ struct RowArgs {
     pr_prod_aux* aux;
     int out_f64;
     Workspace ws;
+};
+
+struct RowGroupArgs {
+    const void* x;
+    int64_t rows, cols;  // 0 < cols < 2^30
+    int shift;           // x's element offset from the previous 32-byte boundary
+    int gl;              // log2 of the lanes per row: 0..5, or 8 (a block per row)
+    void* out;
+    int64_t* argidx;
+    pr_prod_aux* aux;
 };
 
 struct BwdArgs {
@@ -585,6 +609,110 @@ __global__ void __launch_bounds__(MaxBlock<T>::value) k_rows(RowArgs a) {
             }
         }
         v = pend;
+    }
+}
+
+// ------------------------------------------------------------------------
+// Runs of x reduced by groups of lanes
+// ------------------------------------------------------------------------
+
+// Accumulators a lane keeps: one per load in flight where an accumulator is
+// one or two words (shorter chains of dependent operations, and a smaller sum
+// of rounding errors), else one.
+template <class T, int U>
+struct GroupAccs {
+    static constexpr int value = sizeof(typename T::Acc) <= 8 ? U : 1;
+};
+
+// The elements [p0, p0 + len) of x that lane t of G neighbours takes, combined
+// into one Part (indices given to the trait are relative to p0).  The run is
+// covered by 32-byte vectors on the 32-byte grid of memory, lane t taking
+// vectors t, t + G, ..., U of them in flight; of the vectors that hold the
+// run's ends the elements outside it are dropped, and one that is not wholly
+// inside [X0, X1), the elements the caller vouches for, is read element by
+// element.
+template <class T, int U>
+__device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In* x, int64_t p0, int len, int shift,
+                                                       int64_t X0, int64_t X1, int t, int G) {
+    using Ld = typename T::Ld;
+    using E = typename Ld::E;
+    constexpr int VE = kGroupVec / Ld::ES;
+    constexpr int NA = GroupAccs<T, U>::value;
+    // an fp32 accumulator whose Part is a double (FP64_COMBINE) joins it after
+    // every U vectors: a lane here adds more vectors than a thread of a wide
+    // block does, and the mode is there to keep fp32 chains short
+    constexpr bool kWide = sizeof(typename T::Acc) == 4 && sizeof(typename T::Part) == 8;
+    typename T::Part wide = T::part_init();
+    typename T::Acc acc[NA];
+#pragma unroll
+    for (int u = 0; u < NA; u++) acc[u] = T::init();
+    const int mis = (int)((p0 + shift) & (VE - 1));       // elements of the first vector before the run
+    const int nv = len > 0 ? (len + mis + VE - 1) / VE : 0;
+    const char* base = reinterpret_cast<const char*>(x) + (p0 - mis) * Ld::ES;
+    // run-relative element range that whole vectors may be read from
+    const int64_t s0 = X0 - p0, s1 = X1 - p0;
+    const int c_lo = s0 < -VE ? -VE : (int)s0, c_hi = s1 < (int64_t)len + VE ? (int)s1 : len + VE;
+    for (int j = t; j < nv; j += U * G) {
+        Words<kGroupVec> w[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int v = j + u * G, c = v * VE - mis;
+            if (v < nv && c >= c_lo && c + VE <= c_hi) w[u] = ldv<kGroupVec>(base + (int64_t)v * kGroupVec);
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int v = j + u * G, c = v * VE - mis;
+            typename T::Acc& a = acc[u % NA];
+            if (v >= nv) continue;
+            if (c >= 0 && c + VE <= len) {
+                E e[VE];
+                Ld::template dec<kGroupVec>(w[u], e);
+                T::add_vec(a, e, c);
+            } else if (c >= c_lo && c + VE <= c_hi) {
+                E e[VE];
+                Ld::template dec<kGroupVec>(w[u], e);
+#pragma unroll
+                for (int k = 0; k < VE; k++)
+                    if ((unsigned)(c + k) < (unsigned)len) T::add(a, e[k], c + k);
+            } else {
+                const int e1 = c + VE < len ? c + VE : len;
+                for (int i = c > 0 ? c : 0; i < e1; i++) T::add(a, Ld::one(x, p0 + i), i);
+            }
+        }
+        if constexpr (kWide) {
+            wide = T::combine(wide, fold<T, NA>(acc));
+#pragma unroll
+            for (int u = 0; u < NA; u++) acc[u] = T::init();
+        }
+    }
+    return kWide ? wide : fold<T, NA>(acc);
+}
+
+// Combine across the lanes of each group of 2^gl neighbours (gl <= 5; all 32
+// lanes call); every lane of a group gets its result.
+template <class T>
+__device__ __forceinline__ typename T::Part group_combine(typename T::Part p, int gl) {
+    if (gl == 5) return T::warp_reduce(p);
+    for (int m = (1 << gl) >> 1; m >= 1; m >>= 1) p = T::combine(p, shfl_xor_any(p, m));
+    return p;
+}
+
+template <class T>
+__global__ void __launch_bounds__(kGroupBlock) k_rows_group(RowGroupArgs a) {
+    using GR = GridR<T>;
+    using G = typename GR::Part;
+    const auto* x = static_cast<const typename T::Ld::In*>(a.x);
+    const int lanes = 1 << a.gl;
+    const int t = threadIdx.x & (lanes - 1);
+    const int64_t r = ((int64_t)blockIdx.x * kGroupBlock + threadIdx.x) >> a.gl;
+    const bool has = r < a.rows;
+    typename T::Part p = group_part<T, 4>(x, has ? r * a.cols : 0, has ? (int)a.cols : 0, a.shift, 0, a.rows * a.cols,
+                                          t, lanes);
+    p = a.gl > 5 ? block_combine<T>(p) : group_combine<T>(p, a.gl);
+    if (t == 0 && has) {
+        const G g = GR::up(p);
+        GR::store(a.out, r, g, false);
+        GR::store_aux(a.argidx, a.aux, r, g, 0);
     }
 }
 

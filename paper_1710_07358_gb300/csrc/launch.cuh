@@ -24,6 +24,12 @@ cudaError_t launch_rows(const RowArgs& a, int grid, int block, cudaStream_t st) 
     return cudaGetLastError();
 }
 
+template <class T>
+cudaError_t launch_rows_group(const RowGroupArgs& a, int grid, int block, cudaStream_t st) {
+    k_rows_group<T><<<grid, block, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
 template <class T, int U, int VB>
 cudaError_t launch_axis(const AxisArgs& a, int grid, int block, cudaStream_t st) {
     k_axis<T, U, VB><<<grid, block, 0, st>>>(a);
@@ -89,6 +95,9 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
     reg_one<T, 4, 16>(dtype, op, prec, aux, plain, seg);
     reg_one<T, 4, 32>(dtype, op, prec, aux, plain, seg);
     if (seg) {
+        reg_add(KernelKey{K_ROWS_GROUP, dtype, op, prec, aux, 0, 0},
+                KernelEntry{reinterpret_cast<const void*>(&k_rows_group<T>),
+                            reinterpret_cast<void*>(&launch_rows_group<T>)});
         reg_axis<T, 2, 0>(dtype, op, prec, aux);
         reg_axis<T, 2, 16>(dtype, op, prec, aux);
         reg_axis<T, 2, 32>(dtype, op, prec, aux);

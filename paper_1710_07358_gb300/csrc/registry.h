@@ -11,6 +11,7 @@ namespace pr {
 struct ReduceArgs;
 struct SegArgs;
 struct RowArgs;
+struct RowGroupArgs;
 struct AxisArgs;
 struct AxisBwdArgs;
 struct ScanArgs;
@@ -19,7 +20,8 @@ struct BwdArgs;
 enum Kind : uint8_t {
     K_REDUCE = 0, K_SEGMENTED = 1, K_BACKWARD = 2, K_COMBINE = 3, K_ROWS = 4,
     K_AXIS = 5, K_AXIS_FINISH = 6, K_AXIS_EMPTY = 7, K_AXIS_BACKWARD = 8, K_SCAN = 9,
-    K_REDUCE_TAIL = 10  // k_reduce with claimed tail tiles (large inputs)
+    K_REDUCE_TAIL = 10, // k_reduce with claimed tail tiles (large inputs)
+    K_ROWS_GROUP = 11   // a group of lanes per row (short rows, any alignment)
 };
 enum Aux : uint8_t { AUX_NONE = 0, AUX_ARG = 1, AUX_PROD = 2 };
 
@@ -31,6 +33,7 @@ struct KernelKey {
 using ReduceLaunch = cudaError_t (*)(const ReduceArgs&, int grid, int block, cudaStream_t);
 using SegLaunch = cudaError_t (*)(const SegArgs&, int grid, int block, cudaStream_t);
 using RowLaunch = cudaError_t (*)(const RowArgs&, int grid, int block, cudaStream_t);
+using RowGroupLaunch = cudaError_t (*)(const RowGroupArgs&, int grid, int block, cudaStream_t);
 using AxisLaunch = cudaError_t (*)(const AxisArgs&, int grid, int block, cudaStream_t);
 using AxisBwdLaunch = cudaError_t (*)(const AxisBwdArgs&, int grid, int block, cudaStream_t);
 using ScanLaunch = cudaError_t (*)(const ScanArgs&, int grid, int block, size_t smem, cudaStream_t);
