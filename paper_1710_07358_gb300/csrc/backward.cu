@@ -18,6 +18,7 @@
 
 namespace pr {
 
+constexpr int kFlatBlock = 256;
 
 template <class F, int VB>
 __device__ __forceinline__ void st_vec(F* p, const F (&v)[VB / sizeof(F)]);
@@ -128,6 +129,131 @@ __global__ void __launch_bounds__(1024) k_backward(BwdArgs a) {
             }
         }
     }
+}
+
+// Flat form: gi as one array of vectors whatever the rows, for rows too short
+// to fill a chunk of k_backward (which gives a block of 512 threads to every
+// row, however short).  A block takes kFlatU vectors a thread of neighbouring
+// memory; one 64-bit division places the block's first element, a 32-bit
+// multiply-high each vector's (row_inv: floor((2^32 - 1) / cols), whose
+// estimate is at most one short).  A vector that lies in one row takes that
+// row's gradient as k_backward does; one that crosses row ends is filled
+// element by element.  OPK: 0 sum, 1 max/min, 2 prod.
+constexpr int kFlatU = 4;
+constexpr int kFlatVec = 32;
+
+template <class F, int OPK>
+__device__ __forceinline__ RowGrad<F> flat_row(const BwdArgs& a, int64_t r) {
+    const F g = __ldg(static_cast<const F*>(a.g) + r);
+    RowGrad<F> rg{g, -2, false};
+    if constexpr (OPK == 1) {
+        rg.hot = __ldg(a.argidx + r);
+        if (rg.hot < 0) rg.hot = -1;
+    } else if constexpr (OPK == 2) {
+        const pr_prod_aux ax = a.aux[r];
+        rg.gv = ax.zero_count >= 2 ? (F)0 : (F)((double)g * ax.p_nz);
+        rg.div = ax.zero_count == 0;
+        rg.hot = ax.zero_count == 1 ? ax.first_zero : -1;
+    }
+    return rg;
+}
+
+template <class F, int OPK>
+__global__ void __launch_bounds__(kFlatBlock) k_backward_flat(BwdArgs a, unsigned row_inv, int xvec) {
+    constexpr int VE = kFlatVec / (int)sizeof(F);
+    F* gi = static_cast<F*>(a.gi);
+    const F* x = static_cast<const F*>(a.x);
+    const int64_t total = a.rows * a.cols;
+    const int cols = (int)a.cols;
+    const int64_t b0 = (int64_t)blockIdx.x * (kFlatBlock * kFlatU * VE) - a.shift;   // block's first element
+    const int64_t R0 = b0 > 0 ? b0 / a.cols : 0;
+    const int C0 = (int)(b0 - R0 * a.cols);            // its column (negative before gi's first element)
+#pragma unroll
+    for (int u = 0; u < kFlatU; u++) {
+        const int off = (u * kFlatBlock + (int)threadIdx.x) * VE;
+        const int64_t e0 = b0 + off;
+        if (e0 >= total) break;
+        const int ce = C0 + off;
+        int q = ce > 0 ? (int)__umulhi((unsigned)ce, row_inv) : 0;
+        if (ce - q * cols >= cols) q++;
+        int64_t r = R0 + q;
+        int c = ce - q * cols;
+        F vals[VE];
+        if (c >= 0 && c + VE <= cols) {
+            const RowGrad<F> rg = flat_row<F, OPK>(a, r);
+            if constexpr (OPK == 0) {
+#pragma unroll
+                for (int k = 0; k < VE; k++) vals[k] = rg.gv;
+            } else {
+                if (OPK == 2 && rg.div) {
+                    F xe[VE];
+                    if (xvec) {
+                        const Words<kFlatVec> w = ldv<kFlatVec>(x + e0);
+                        memcpy(xe, w.w, kFlatVec);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < VE; k++) xe[k] = __ldg(x + e0 + k);
+                    }
+#pragma unroll
+                    for (int k = 0; k < VE; k++) vals[k] = rg.gv / xe[k];
+                } else {
+                    const int64_t h = rg.hot - c;
+                    const int hk = (h >= 0 && h < VE) ? (int)h : -1;
+#pragma unroll
+                    for (int k = 0; k < VE; k++) vals[k] = hk == k ? rg.gv : (F)0;
+                }
+            }
+            st_vec<F, kFlatVec>(gi + e0, vals);
+            continue;
+        }
+        RowGrad<F> rg{};
+        bool have = false;
+#pragma unroll
+        for (int k = 0; k < VE; k++) {
+            vals[k] = (F)0;
+            if (c == cols) {
+                c = 0;
+                r++;
+                have = false;
+            }
+            if (c >= 0 && r < a.rows) {
+                if (!have) rg = flat_row<F, OPK>(a, r);
+                have = true;
+                vals[k] = OPK == 0 ? rg.gv : (rg.div ? rg.gv / __ldg(x + e0 + k) : (rg.hot == c ? rg.gv : (F)0));
+            }
+            c++;
+        }
+        if (e0 >= 0 && e0 + VE <= total) {
+            st_vec<F, kFlatVec>(gi + e0, vals);
+        } else {
+#pragma unroll
+            for (int k = 0; k < VE; k++)
+                if (e0 + k >= 0 && e0 + k < total) gi[e0 + k] = vals[k];
+        }
+    }
+}
+
+template <class F, int OPK>
+static void flat_go(const BwdArgs& a, int64_t grid, bool xvec, cudaStream_t st) {
+    k_backward_flat<F, OPK><<<(unsigned)grid, kFlatBlock, 0, st>>>(a, 0xffffffffu / (unsigned)a.cols, xvec ? 1 : 0);
+}
+
+// shift in a is gi's element offset from the previous 32-byte boundary
+template <class F>
+static cudaError_t launch_flat(const BwdArgs& a, cudaStream_t st) {
+    constexpr int64_t VE = kFlatVec / (int)sizeof(F);
+    const int64_t per = kFlatBlock * kFlatU * VE;
+    const int64_t grid = (a.rows * a.cols + a.shift + per - 1) / per;
+    if (grid > 0x7fffffff) return cudaErrorInvalidConfiguration;
+    const bool xvec = ((uintptr_t)a.x - (uintptr_t)a.gi) % kFlatVec == 0;
+    if (a.op == PR_SUM) flat_go<F, 0>(a, grid, xvec, st);
+    else if (a.op == PR_PROD) flat_go<F, 2>(a, grid, xvec, st);
+    else flat_go<F, 1>(a, grid, xvec, st);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_backward_flat(const BwdArgs& a, bool f64, cudaStream_t st) {
+    return f64 ? launch_flat<double>(a, st) : launch_flat<float>(a, st);
 }
 
 template <class F, int U, int VB>

@@ -55,6 +55,9 @@ const KernelEntry* reg_find(const KernelKey& k);
 constexpr int kUnrolls[] = {2, 4};
 constexpr int kVecBytes[] = {16, 32};
 
+// Flat gradient of a row reduction (backward.cu); a.shift counts from the previous 32-byte boundary.
+cudaError_t launch_backward_flat(const BwdArgs& a, bool f64, cudaStream_t st);
+
 void register_f32();
 void register_f32_seg();
 void register_f16();

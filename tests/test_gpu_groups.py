@@ -1,12 +1,12 @@
-"""Rows reduced by groups of lanes (short rows, any length and alignment): every
-form the rule sends there against the general segmented path and the oracle,
-at the edges of vectors and groups."""
+"""Rows reduced by groups of lanes (short rows, any length and alignment), and
+the flat gradient of short rows: every form the rule sends there against the
+general segmented path and the oracle, at the edges of vectors and groups."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_1710_07358_gb300 import pr, synth
-from gpu_helpers import guarded_like, prod_rel_bound, same_float, sum_bound, to_device, values_of
+from gpu_helpers import Guarded, guarded_like, prod_rel_bound, same_float, sum_bound, to_device, values_of
 
 pytestmark = pytest.mark.gpu
 
@@ -115,3 +115,39 @@ def test_rows_by_groups_special_values():
                 assert same_float(vals[r], v) and int(idx[r]) == i, (op, offset, r)
     s = pr.reduce_rows(to_device(x.reshape(-1), "f32", 1).view(rows, cols), "sum")
     assert torch.isnan(s[2]) and torch.isnan(s[3]) and float(s[4]) == -np.inf and float(s[5]) == np.inf
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("op", ["sum", "max", "prod"])
+@pytest.mark.parametrize("rows,cols", [(1, 1), (3000, 1), (1000, 2), (777, 7), (1000, 8), (301, 33), (5, 2047), (3, 8193)])
+def test_flat_gradient(dtype, op, rows, cols):
+    """Bit for bit the rules' own float expressions, at every alignment of
+    grad_in and with x aligned like it or not."""
+    import torch
+    np_t = np.float32 if dtype == "f32" else np.float64
+    x = (1 + 0.1 * synth.normal_f32(rows * cols, rows + cols)).astype(np_t).reshape(rows, cols)
+    if op == "prod":                       # rows without, with one and with two zeros
+        x[1::3, 0] = 0
+        x[2::3, -1] = 0
+        x[2::3, 0] = 0
+    g = synth.normal_f32(rows, 3).astype(np_t)
+    gt = torch.from_numpy(g).cuda()
+    for off_x, off_g in ((0, 0), (1, 1), (0, 3)):
+        t = to_device(x.reshape(-1), dtype, off_x).view(rows, cols)
+        _, more = pr.reduce_rows(t, op, argidx=op == "max", aux=op == "prod") if op != "sum" else (None, None)
+        buf = Guarded(rows * cols + off_g, t.dtype, fill=7)
+        gi = buf.tensor[off_g:]
+        pr.reduce_backward(op, t, gt, argidx=more if op == "max" else None, aux=more if op == "prod" else None, out=gi)
+        buf.check()
+        assert bool((buf.tensor[:off_g] == 7).all())
+        if op == "sum":
+            want = np.broadcast_to(g[:, None], x.shape)
+        elif op == "max":
+            want = np.where(np.arange(cols) == x.argmax(1)[:, None], g[:, None], np_t(0))
+        else:
+            p_nz, zc, zi = (v.cpu().numpy() for v in pr.prod_aux_fields(more))
+            gp = (g.astype(np.float64) * p_nz).astype(np_t)[:, None]
+            zc, zi = zc[:, None], zi[:, None]
+            with np.errstate(divide="ignore"):
+                want = np.where(zc == 0, gp / x, np.where((zc == 1) & (np.arange(cols) == zi), gp, np_t(0)))
+        assert np.array_equal(gi.cpu().numpy().reshape(rows, cols), want), (off_x, off_g)
