@@ -106,7 +106,8 @@ typedef struct {
 } pr_config;
 
 /* Kernel families with their own configurations: REDUCE (pr_reduce*),
- * SEGMENTED (pr_segmented_reduce*, and rows that do not fit ROWS), BACKWARD
+ * SEGMENTED (pr_segmented_reduce* of fewer than 8192 segments, 512 with argidx
+ * or aux, and rows that do not fit ROWS; more segments ignore it), BACKWARD
  * (pr_reduce_backward), ROWS (pr_reduce_rows for few long rows when cols is a
  * whole number of vectors and x is aligned to the vector width; bucketed by
  * rows*cols; shorter or more rows ignore it: groups of lanes take a row each), AXIS

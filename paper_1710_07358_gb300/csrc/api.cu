@@ -167,7 +167,9 @@ static pr_status device_info(DevInfo* out, int* dev_out) {
     return PR_OK;
 }
 
-static size_t ws_bytes(int gmax) { return (size_t)3 * gmax * kSlot + (size_t)(gmax + 64) * 4; }
+static size_t ws_bytes(int gmax) {
+    return (size_t)3 * gmax * kSlot + (size_t)(gmax + 64) * 4 + kSegTasks * sizeof(SegTask);
+}
 
 static pr_status get_ws(cudaStream_t st, Workspace* out) {
     DevInfo di;
@@ -206,6 +208,8 @@ static pr_status get_ws(cudaStream_t st, Workspace* out) {
     ws.blk_done = u + gmax + 2;
     ws.err = reinterpret_cast<int*>(u + gmax + 32);
     ws.gmax = gmax;
+    ws.task_count = u + gmax + 3;
+    ws.tasks = reinterpret_cast<SegTask*>(u + gmax + 64);   // (16-byte aligned: gmax is a multiple of 32)
     g_ws[key] = WsRec{ws, base, bytes};
     *out = ws;
     return PR_OK;
@@ -469,6 +473,47 @@ static void seg_split(int64_t nseg, int grid, int gmax, int* chunks_per_block, i
         *chunks_per_block = 1;
         *dynamic = 0;
     }
+}
+
+// k_seg_group and k_seg_long are a pair that shares the stream's task list, as
+// k_axis and k_axis_finish share its partials: they are enqueued together,
+// whatever other host threads enqueue.
+static std::mutex g_pair_mu;
+
+static pr_status run_seg_group(const void* x, const int64_t* off, int64_t nseg, int dtype, int op, int prec, int aux,
+                               void* out, int64_t* argidx, pr_prod_aux* paux, cudaStream_t st) {
+    const KernelEntry* e = reg_find(KernelKey{K_SEG_GROUP, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux, 0, 0});
+    const KernelEntry* el = reg_find(KernelKey{K_SEG_LONG, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux, 0, 0});
+    if (!e || !el)
+        return fail(PR_ERR_UNSUPPORTED, "no segmented kernel for dtype %d op %d precision %d aux %d", dtype, op, prec, aux);
+    DevInfo di;
+    pr_status s = device_info(&di, nullptr);
+    if (s != PR_OK) return s;
+    Workspace ws;
+    s = get_ws(st, &ws);
+    if (s != PR_OK) return s;
+    int occ = 0, occ_l = 0;
+    if ((s = occupancy(e->fn, kSegBlock, &occ)) != PR_OK) return s;
+    if ((s = occupancy(el->fn, kGroupBlock, &occ_l)) != PR_OK) return s;
+    if (occ < 1 || occ_l < 1) return fail(PR_ERR_UNSUPPORTED, "segmented kernels cannot run");
+    const int64_t need = (nseg + kSegBlock / 32 - 1) / (kSegBlock / 32);   // a segment a warp at least
+    const int64_t most = (int64_t)di.sms * occ;
+    // partials go by task index into head and tail
+    const size_t room = (size_t)2 * ws.gmax * kSlot / (size_t)e->part_bytes;
+    SegGroupArgs a{x, off, nseg, (int)(reinterpret_cast<uintptr_t>(x) % kGroupVec) / elem_size(dtype),
+                   room < kSegTasks ? (unsigned)room : kSegTasks, out, argidx, paux, ws};
+    std::lock_guard<std::mutex> lk(g_pair_mu);
+    PR_INJECT_LAUNCH();
+    cudaError_t err = reinterpret_cast<SegGroupLaunch>(e->launch)(a, (int)(need < most ? need : most), kSegBlock, st);
+    if (err != cudaSuccess) return fail(PR_ERR_CUDA, "segmented launch: %s", cudaGetErrorString(err));
+    const bool injected = inject(PR_FAULT_LAUNCH);
+    if (!injected) err = reinterpret_cast<SegGroupLaunch>(el->launch)(a, di.sms * occ_l, kGroupBlock, st);
+    if (injected || err != cudaSuccess) {
+        cudaMemsetAsync(ws.task_count, 0, sizeof(unsigned), st);   // the list is for this call only
+        if (injected) return fail(PR_ERR_CUDA, "kernel launch failed (injected by the test hook)");
+        return fail(PR_ERR_CUDA, "segmented launch: %s", cudaGetErrorString(err));
+    }
+    return PR_OK;
 }
 
 static pr_status run_segmented(const void* x, const int64_t* off, int64_t cols, int64_t nseg, int dtype, int op,
@@ -994,6 +1039,8 @@ pr_status pr_reduce_rows(const void* x, int64_t rows, int64_t cols, pr_dtype dty
         const int auxk = argidx ? AUX_ARG : (aux ? AUX_PROD : AUX_NONE);
         pr_status s = run_rows_group(x, rows, cols, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream);
         if (s != PR_ERR_UNSUPPORTED) return s;
+    if (offsets && nseg >= (auxk == AUX_NONE ? kSegGroupMin : kSegGroupMinHeavy))
+        return run_seg_group(x, offsets, nseg, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream);
         const pr_config c = lookup_cfg(PR_KIND_ROWS, dtype, op, precision, rows * cols);
         s = run_rows(x, rows, cols, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream, c);
         if (s != PR_ERR_UNSUPPORTED) return s;

@@ -41,6 +41,18 @@
 //   order.  Partials are indexed by chunk, not by block, so results are
 //   deterministic for a fixed launch configuration whatever the claim order.
 //
+// k_seg_group, k_seg_long  segments of a CSR offsets array when there are many
+//   (kSegGroupMin): a tile of k_segmented costs its block several barriers and
+//   a search, which hundreds of short segments a tile do not pay for.  The
+//   first kernel takes up to 32 neighbouring segments a warp, through shared
+//   memory where they are short; the second shares the long ones among all
+//   warps, chunk by chunk.  fp32 sum on GB300: 10^6 segments of 24 elements on
+//   average (96 MB) 841 -> 52 us (0.30 of a 6.8 TB/s copy), 65536 of 1000 230
+//   -> 64, 10^5 log-uniform to 16384 316 -> 202, 8192 of 40000 207 -> 207;
+//   maximum with index of the first 976 -> 107, of the last 538 -> 243.  Short
+//   segments are bound by instructions, about 24 warp instructions a segment
+//   of 24 (ncu: issue slots 60 % busy, no one stall dominant), long ones by HBM.
+//
 // k_rows       equal rows of `cols` elements (cols a multiple of the vector
 //   width, x aligned to it): the flattened vectors are split into one run of
 //   whole tiles per block; a block streams its run exactly like k_reduce and
@@ -72,9 +84,36 @@ namespace pr {
 
 constexpr int kSlot = 64;      // bytes per partial slot (>= sizeof(Part) of every trait)
 constexpr int kSmallSeg = 512; // segments up to this length are reduced by one warp
+// Segmented launches of this many segments and more take k_seg_group and
+// k_seg_long; smaller ones k_segmented, which hands segments over to groups of
+// lanes itself when their mean is at most kGroupMean and none is longer than
+// kGroupMost elements (which every block sees for itself: no second launch).
+// Measured on GB300 (us, fp32 sum, k_segmented before / k_segmented with the
+// hand-over / k_seg_group + k_seg_long): 1000 segments of 24 on average 72 /
+// 6.4 / 8.5, 4096 log-uniform to 4096 22.5 / 12.7 / 18.5, 10^4 of 24 98 / 25 /
+// 8.5; k_segmented splits few and long ones best (64 log-uniform to 2^20 16 /
+// 16 / 25, 4096 to 2^20 183 / 183 / 189) unless the accumulator is heavy
+// (maximum with index: 4096 to 2^20 416 / 417 / 218, 877 to 380 000 76 / 76 /
+// 50, 64 to 2^20 31 / 32 / 30).
+constexpr int64_t kSegGroupMin = 8192;
+constexpr int64_t kSegGroupMinHeavy = 512;   // kernels with an index or product state
+constexpr int64_t kGroupMean = 4096;
+constexpr int64_t kGroupMost = 8192;
 constexpr int kGroupBlock = 256;   // threads per block of the group kernels
 constexpr int kGroupVec = 32;      // bytes per vector load
 enum : int { kErrInvalid = 1, kErrTimeout = 4 };
+
+// One task of k_seg_group's shared part: a long segment, or a chunk of one
+// that is longer than a chunk.  A segment's tasks follow one another; its
+// partials and its count of finished chunks go by task index.
+struct SegTask {
+    int64_t seg;
+    unsigned first;      // the segment's first task
+    unsigned finished;   // in the first task: chunks whose partials are stored
+};
+
+// Tasks that a launch lists at most, as far as the partial slots suffice.
+constexpr unsigned kSegTasks = 65536;
 
 struct Workspace {
     char* partials;      // gmax slots (k_reduce)
@@ -86,6 +125,8 @@ struct Workspace {
     unsigned* blk_done;  // blocks finished (k_segmented), zero between launches
     int* err;            // device error word
     int gmax;
+    SegTask* tasks = nullptr;       // kSegTasks (k_seg_group)
+    unsigned* task_count = nullptr; // tasks listed, zero between launches
 };
 
 struct ReduceArgs {
@@ -125,6 +166,18 @@ struct RowArgs {
     int64_t* argidx;
     pr_prod_aux* aux;
     int out_f64;
+    Workspace ws;
+};
+
+struct SegGroupArgs {
+    const void* x;
+    const int64_t* off;  // nseg+1 CSR offsets
+    int64_t nseg;
+    int shift;           // x's element offset from the previous 32-byte boundary
+    unsigned tasks;      // tasks that may be listed: kSegTasks, or what the partial slots hold
+    void* out;
+    int64_t* argidx;
+    pr_prod_aux* aux;
     Workspace ws;
 };
 
@@ -624,8 +677,52 @@ struct GroupAccs {
     static constexpr int value = sizeof(typename T::Acc) <= 8 ? U : 1;
 };
 
+// An fp32 accumulator whose Part is a double (FP64_COMBINE).  A lane of a
+// group adds more elements than a thread of a wide block does, and the mode
+// is there to keep fp32 chains short, so groups join it to the double part
+// often: after every few vectors of long runs, after every element of short
+// ones.
+template <class T>
+constexpr bool kWidePart = sizeof(typename T::Acc) == 4 && sizeof(typename T::Part) == 8;
+
+// Accumulation of a short run, an element or a few neighbours at a time.
+template <class T>
+struct ShortAcc {
+    using A = std::conditional_t<kWidePart<T>, typename T::Part, typename T::Acc>;
+    A a;
+    __device__ __forceinline__ ShortAcc() {
+        if constexpr (kWidePart<T>) a = T::part_init();
+        else a = T::init();
+    }
+    __device__ __forceinline__ void add(typename T::Ld::E e, int i) {
+        if constexpr (kWidePart<T>) {
+            typename T::Acc one = T::init();
+            T::add(one, e, i);
+            a = T::combine(a, T::to_part(one));
+        } else {
+            T::add(a, e, i);
+        }
+    }
+    // N elements with indices from i on, summed as a tree (a trait without
+    // indices takes any N elements)
+    template <int N>
+    __device__ __forceinline__ void add_vec(const typename T::Ld::E (&e)[N], int i) {
+        if constexpr (kWidePart<T>) {
+            typename T::Acc one = T::init();
+            T::add_vec(one, e, i);
+            a = T::combine(a, T::to_part(one));
+        } else {
+            T::add_vec(a, e, i);
+        }
+    }
+    __device__ __forceinline__ typename T::Part part() const {
+        if constexpr (kWidePart<T>) return a;
+        else return T::to_part(a);
+    }
+};
+
 // The elements [p0, p0 + len) of x that lane t of G neighbours takes, combined
-// into one Part (indices given to the trait are relative to p0).  The run is
+// into one Part (the trait is given indices relative to p0, plus i0).  The run is
 // covered by 32-byte vectors on the 32-byte grid of memory, lane t taking
 // vectors t, t + G, ..., U of them in flight; of the vectors that hold the
 // run's ends the elements outside it are dropped, and one that is not wholly
@@ -633,15 +730,11 @@ struct GroupAccs {
 // element.
 template <class T, int U>
 __device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In* x, int64_t p0, int len, int shift,
-                                                       int64_t X0, int64_t X1, int t, int G) {
+                                                       int64_t X0, int64_t X1, int t, int G, int64_t i0 = 0) {
     using Ld = typename T::Ld;
     using E = typename Ld::E;
     constexpr int VE = kGroupVec / Ld::ES;
     constexpr int NA = GroupAccs<T, U>::value;
-    // an fp32 accumulator whose Part is a double (FP64_COMBINE) joins it after
-    // every U vectors: a lane here adds more vectors than a thread of a wide
-    // block does, and the mode is there to keep fp32 chains short
-    constexpr bool kWide = sizeof(typename T::Acc) == 4 && sizeof(typename T::Part) == 8;
     typename T::Part wide = T::part_init();
     typename T::Acc acc[NA];
 #pragma unroll
@@ -667,25 +760,26 @@ __device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In*
             if (c >= 0 && c + VE <= len) {
                 E e[VE];
                 Ld::template dec<kGroupVec>(w[u], e);
-                T::add_vec(a, e, c);
+                T::add_vec(a, e, i0 + c);
             } else if (c >= c_lo && c + VE <= c_hi) {
                 E e[VE];
                 Ld::template dec<kGroupVec>(w[u], e);
 #pragma unroll
                 for (int k = 0; k < VE; k++)
-                    if ((unsigned)(c + k) < (unsigned)len) T::add(a, e[k], c + k);
+                    if ((unsigned)(c + k) < (unsigned)len) T::add(a, e[k], i0 + c + k);
             } else {
                 const int e1 = c + VE < len ? c + VE : len;
-                for (int i = c > 0 ? c : 0; i < e1; i++) T::add(a, Ld::one(x, p0 + i), i);
+                for (int i = c > 0 ? c : 0; i < e1; i++) T::add(a, Ld::one(x, p0 + i), i0 + i);
             }
         }
-        if constexpr (kWide) {
+        if constexpr (kWidePart<T>) {
             wide = T::combine(wide, fold<T, NA>(acc));
 #pragma unroll
             for (int u = 0; u < NA; u++) acc[u] = T::init();
         }
     }
-    return kWide ? wide : fold<T, NA>(acc);
+    if constexpr (kWidePart<T>) return wide;
+    else return fold<T, NA>(acc);
 }
 
 // Combine across the lanes of each group of 2^gl neighbours (gl <= 5; all 32
@@ -695,6 +789,93 @@ __device__ __forceinline__ typename T::Part group_combine(typename T::Part p, in
     if (gl == 5) return T::warp_reduce(p);
     for (int m = (1 << gl) >> 1; m >= 1; m >>= 1) p = T::combine(p, shfl_xor_any(p, m));
     return p;
+}
+
+// Lanes per segment (log2) for segments of `mean` elements on average: two
+// loads a lane for half as many vectors again as such a segment touches, so
+// that most segments of a spread of lengths need one round of loads.
+template <class Ld>
+__device__ __forceinline__ int group_lanes(int64_t mean) {
+    const int64_t nv = mean / (kGroupVec / Ld::ES) + 1;
+    int gl = 0;
+    while (gl < 5 && ((int64_t)2 << gl) < nv + nv / 2) gl++;
+    return gl;
+}
+
+// The result of segment s, from the lane that holds it.
+template <class T>
+__device__ __forceinline__ void store_segment(const typename T::Part& p, int64_t s, void* out, int64_t* argidx,
+                                              pr_prod_aux* aux) {
+    using GR = GridR<T>;
+    const typename GR::Part g = GR::up(p);
+    GR::store(out, s, g, false);
+    GR::store_aux(argidx, aux, s, g, 0);
+}
+
+// One warp reduces up to 32 neighbouring segments s0, s0 + 1, ...: lane i
+// holds segment s0 + i's first element b and its length (0: none; the segment
+// lies in [X0, X1)).  Groups of 2^gl lanes take a segment each, in rounds,
+// two loads a lane at a time; the vectors that hold a segment's ends are
+// masked.  A segment of more than four loads a lane would hold the other
+// groups up and waits for the whole warp, after the rounds; so do all where
+// a vector might not lie in [X0, X1).
+template <class T>
+__device__ __forceinline__ void warp_segments(const typename T::Ld::In* x, int shift, int64_t X0, int64_t X1, int64_t s0,
+                                              int64_t b, int len, int gl, void* out, int64_t* argidx,
+                                              pr_prod_aux* aux) {
+    using Ld = typename T::Ld;
+    using E = typename Ld::E;
+    using Part = typename T::Part;
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int VE = kGroupVec / Ld::ES;
+    constexpr int U = 2;
+    const int lane = threadIdx.x & 31, lanes = 1 << gl, t = lane & (lanes - 1);
+    const int per = 32 >> gl;                                // segments a round
+    const bool one = len > 0 && len <= (4 * VE << gl) && b - VE >= X0 && b + len + VE <= X1;
+    unsigned rounds = gl < 5 ? __ballot_sync(kAll, one) : 0u;
+    unsigned rest = __ballot_sync(kAll, len > 0) & ~rounds;
+    const int small = rounds >> lane & 1u ? len : 0;
+    for (int k = 0; rounds >> k; k += per) {
+        const int i = k + (lane >> gl);
+        const int64_t p0 = __shfl_sync(kAll, b, i);
+        const int n = __shfl_sync(kAll, small, i);
+        const int mis = (int)((p0 + shift) & (VE - 1));
+        const int nv = n > 0 ? (n + mis + VE - 1) / VE : 0;
+        const typename Ld::In* base = x + (p0 - mis);
+        ShortAcc<T> acc;
+        for (int j = t; __any_sync(kAll, j < nv); j += U * lanes) {
+            Words<kGroupVec> w[U];
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (j + u * lanes < nv) w[u] = ldv<kGroupVec>(base + (j + u * lanes) * VE);
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (j + u * lanes >= nv) continue;
+                const int c = (j + u * lanes) * VE - mis;
+                E e[VE];
+                Ld::template dec<kGroupVec>(w[u], e);
+                // bit i: element c + i belongs to the segment
+                const int lo = c < 0 ? -c : 0, hi = n - c;
+                const unsigned m = (hi >= VE ? (unsigned)((1ull << VE) - 1) : (1u << hi) - 1u) >> lo << lo;
+                if (c >= 0 && hi >= VE) {
+                    acc.add_vec(e, c);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < VE; q++)
+                        if (m >> q & 1u) acc.add(e[q], c + q);
+                }
+            }
+        }
+        const Part p = group_combine<T>(acc.part(), gl);
+        if (t == 0 && n > 0) store_segment<T>(p, s0 + i, out, argidx, aux);
+        if (k + per >= 32) break;
+    }
+    for (; rest; rest &= rest - 1) {
+        const int i = __ffs(rest) - 1;
+        const Part p = T::warp_reduce(
+            group_part<T, 2>(x, __shfl_sync(kAll, b, i), __shfl_sync(kAll, len, i), shift, X0, X1, lane, 32));
+        if (lane == 0) store_segment<T>(p, s0 + i, out, argidx, aux);
+    }
 }
 
 template <class T>
@@ -726,10 +907,8 @@ struct Segs {
     __device__ __forceinline__ int64_t raw(int64_t s) const { return off ? __ldg(off + s) : s * cols; }
     // segment bounds clamped to [P0, P1]: malformed offsets cannot move a read
     // outside the range the caller vouches for
-    __device__ __forceinline__ int64_t begin(int64_t s) const {
-        const int64_t b = raw(s);
-        return b < P0 ? P0 : (b > P1 ? P1 : b);
-    }
+    __device__ __forceinline__ int64_t clamp(int64_t b) const { return b < P0 ? P0 : (b > P1 ? P1 : b); }
+    __device__ __forceinline__ int64_t begin(int64_t s) const { return clamp(raw(s)); }
     __device__ __forceinline__ int64_t end(int64_t s) const { return begin(s + 1); }
     // Largest s in [lo, nseg) with begin(s) <= p (requires begin(lo) <= p),
     // found by one warp (all 32 lanes call; every lane gets the answer).
@@ -761,6 +940,29 @@ struct Segs {
         return lo;
     }
 };
+
+// Batches q, q + nwarp, ... of 2^batch neighbouring segments, one a warp at a
+// time (batch <= 5), none longer than `most`.  Empty segments get the
+// identity, malformed offsets raise the error word.
+template <class T>
+__device__ __forceinline__ void segment_batches(const Segs& sg, const typename T::Ld::In* x, int shift, int batch,
+                                                int64_t q, int64_t nwarp, int64_t most, void* out, int64_t* argidx,
+                                                pr_prod_aux* aux, int* err) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nbatch = (sg.nseg + ((int64_t)1 << batch) - 1) >> batch;
+    int gl = group_lanes<typename T::Ld>((sg.P1 - sg.P0) / sg.nseg);
+    if (gl < 5 - batch) gl = 5 - batch;          // a short batch has lanes to spare
+    for (; q < nbatch; q += nwarp) {
+        const int64_t s = (q << batch) + lane;
+        const bool mine = lane < (1 << batch) && s < sg.nseg;
+        const int64_t rb = mine ? sg.raw(s) : 0, re = mine ? sg.raw(s + 1) : 0;
+        if (mine && (rb > re || rb < 0)) atomicOr(err, kErrInvalid);
+        const int64_t b = sg.clamp(rb), len = mine ? sg.clamp(re) - b : 0;
+        if (mine && len == 0) T::store_empty(out, s, false, argidx, aux);
+        warp_segments<T>(x, shift, sg.P0, sg.P1, q << batch, b, len > 0 && len <= most ? (int)len : 0, gl, out, argidx,
+                         aux);
+    }
+}
 
 template <class T, int U, int VB>
 struct SegCtx {
@@ -837,6 +1039,22 @@ __global__ void __launch_bounds__(512) k_segmented(SegArgs a) {
     const int64_t P1 = rawN < P0 ? P0 : rawN;
     sg.P0 = P0;
     sg.P1 = P1;
+
+    // Segments that are all short go to groups of lanes (see k_seg_group; this
+    // kernel has the launches of fewer than kSegGroupMin of them, where every
+    // block can look at all lengths for itself).
+    if (a.off && nseg < kSegGroupMin && P1 - P0 <= nseg * kGroupMean) {
+        bool longer = false;
+        for (int64_t s = threadIdx.x; s < nseg; s += blockDim.x) longer |= sg.end(s) - sg.begin(s) > kGroupMost;
+        if (!__syncthreads_or(longer)) {
+            const int64_t nwarp = nth >> 5;
+            int batch = 5;
+            while (batch > 0 && (nseg >> batch) < nwarp) batch--;
+            segment_batches<T>(sg, x, (int)(reinterpret_cast<uintptr_t>(x) % kGroupVec) / Ld::ES, batch, gtid >> 5,
+                               nwarp, kGroupMost, a.out, a.argidx, a.aux, a.ws.err);
+            return;
+        }
+    }
 
     // Empty segments get the identity; malformed offsets raise the error word.
     for (int64_t s = gtid; s < nseg; s += nth) {
@@ -1036,6 +1254,261 @@ __global__ void __launch_bounds__(512) k_segmented(SegArgs a) {
         __threadfence();
         if (atomicAdd(a.ws.blk_done, 1u) == gridDim.x - 1) {
             *a.ws.chunk_ctr = 0u;
+            *a.ws.blk_done = 0u;
+        }
+    }
+}
+
+// ------------------------------------------------------------------------
+// Many segments
+// ------------------------------------------------------------------------
+
+// A segment of more than `most` elements is left to k_seg_long, in chunks of
+// `chunk`.  Both grow with the elements so that the tasks fit: at most half
+// of them long segments (unless there are that few segments at all), the
+// other half the further chunks of those.
+constexpr int64_t kLongSeg = 2048;
+constexpr int64_t kLongChunk = 8192;
+
+struct SegSplit {
+    int64_t most, chunk;
+};
+__device__ __forceinline__ SegSplit seg_split_lengths(int64_t total, int64_t nseg, unsigned tasks) {
+    const int64_t share = total / (tasks / 2) + 1;
+    const int64_t most = nseg <= tasks / 2 || share < kLongSeg ? kLongSeg : share;
+    const int64_t chunk = share < kLongChunk ? kLongChunk : share;
+    return {most, chunk < most ? most : chunk};
+}
+
+__device__ __forceinline__ Segs seg_bounds(const int64_t* off, int64_t nseg) {
+    Segs sg{off, 0, nseg, 0, 0};
+    const int64_t raw0 = sg.raw(0), rawN = sg.raw(nseg);
+    sg.P0 = raw0 < 0 ? 0 : raw0;
+    sg.P1 = rawN < sg.P0 ? sg.P0 : rawN;
+    return sg;
+}
+
+// 1. All but the long segments, up to 32 neighbours a warp at a time; the
+// long ones are listed as tasks of at most a chunk.
+//
+// Short segments (at most kStageMean bytes on average) are staged: a batch of
+// neighbours is one contiguous run, copied to the warp's shared memory, so
+// that loads are whole and coalesced whatever the lengths, and a group's
+// lanes read their segment element by element, with no vector cut by a
+// segment's end.  A batch that does not fit (or reaches the ends of x, or
+// holds a long segment) is reduced from x directly.  One stage a warp: the
+// other warps of the SM cover its wait, and a second stage would take the
+// shared memory that the L1 cache needs for the loads in flight of the direct
+// path and of k_seg_long (measured: 8192 segments of 40000 254 us with two
+// stages, 207 with one).  Five blocks an SM: 96 registers, the most that no
+// trait on the fp32 path spills at (10^6 segments of 24: 52 us; six blocks 53,
+// eight 53, and 118 against 106 for the maximum with index).
+constexpr int kSegBlock = 128;
+constexpr int kStageBytes = 4096;    // a warp's stage: one batch
+constexpr int kStageMean = 512;
+
+template <class T>
+__global__ void __launch_bounds__(kSegBlock, 5) k_seg_group(SegGroupArgs a) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // k_seg_long may take its place as blocks leave
+    using Ld = typename T::Ld;
+    using In = typename Ld::In;
+    using Part = typename T::Part;
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int VE = kGroupVec / Ld::ES, CAP = kStageBytes / Ld::ES, PE = 16 / Ld::ES;
+    __shared__ __align__(32) unsigned char s_stage[kSegBlock / 32][kStageBytes];
+    const In* x = static_cast<const In*>(a.x);
+    const Segs sg = seg_bounds(a.off, a.nseg);
+    const SegSplit sp = seg_split_lengths(sg.P1 - sg.P0, a.nseg, a.tasks);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t nwarp = (int64_t)gridDim.x * (kSegBlock / 32);
+    const int64_t mean = (sg.P1 - sg.P0) / a.nseg;
+    const bool stage = mean * Ld::ES <= kStageMean;
+    int batch = 5;
+    while (batch > 0 && (a.nseg >> batch) < nwarp) batch--;
+    if (stage)
+        while (batch > 1 && mean << batch > CAP * 3 / 4) batch--;   // (mean <= CAP / 8)
+    const int64_t nbatch = (a.nseg + ((int64_t)1 << batch) - 1) >> batch;
+    int gl = group_lanes<Ld>(mean);
+    if (gl < 5 - batch) gl = 5 - batch;          // a short batch has lanes to spare
+    const In* v = reinterpret_cast<const In*>(s_stage[warp]);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_stage[warp]);
+
+    // this lane's segment of batch w (raw bounds)
+    auto load = [&](int64_t w, int64_t& b, int64_t& e) {
+        const int64_t s = (w << batch) + lane;
+        const bool mine = lane < (1 << batch) && s < a.nseg && w < nbatch;
+        b = mine ? sg.raw(s) : 0;
+        e = mine ? sg.raw(s + 1) : 0;
+    };
+    int64_t q = (int64_t)blockIdx.x * (kSegBlock / 32) + warp;
+    int64_t nb, ne;
+    load(q, nb, ne);
+    for (; q < nbatch; q += nwarp) {
+        const int64_t rb = nb, re = ne, s0 = q << batch;
+        const bool mine = lane < (1 << batch) && s0 + lane < a.nseg;
+        const unsigned in = __ballot_sync(kAll, mine);
+        if (stage) {
+            // well-formed, inside [P0, P1) with the vectors around it, and
+            // short enough: 32-bit places from the first staged element on
+            const int64_t p0 = __shfl_sync(kAll, rb, 0);
+            const int mis = (int)((p0 + a.shift) & (VE - 1));
+            const int64_t base = p0 - mis;
+            const uint64_t ob = (uint64_t)(rb - base), oe = (uint64_t)(re - base);
+            const bool ok = !mine || (ob <= oe && oe <= (uint64_t)(CAP - VE));
+            const int n = __shfl_sync(kAll, (int)oe, 31 - __clz(in));
+            const int pieces = (n + PE - 1) / PE;                                  // 16 bytes each
+            if (__all_sync(kAll, ok) && base >= sg.P0 && base + pieces * PE <= sg.P1) {
+                const char* src = reinterpret_cast<const char*>(x + base);
+                for (int i = lane; i < pieces; i += 32)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 16), "l"(src + i * 16) : "memory");
+                load(q + nwarp, nb, ne);
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncwarp();
+                const int lanes = 1 << gl, t = lane & (lanes - 1);
+                const int r0 = (int)ob, n0 = mine ? (int)oe - r0 : 0;
+                if (mine && n0 == 0) T::store_empty(a.out, s0 + lane, false, a.argidx, a.aux);
+                for (int k = 0; k < 1 << batch; k += 32 >> gl) {
+                    const int i = k + (lane >> gl);
+                    const In* run = v + __shfl_sync(kAll, r0, i);
+                    const int len = __shfl_sync(kAll, n0, i);
+                    ShortAcc<T> acc;
+                    int j = t;
+                    if constexpr (!T::kIdx && !kWidePart<T>) {
+                        // four at a time, summed pairwise: a shorter chain of
+                        // operations and of roundings
+                        for (; j + 3 * lanes < len; j += 4 * lanes) {
+                            const typename Ld::E e[4] = {Ld::lone(run[j]), Ld::lone(run[j + lanes]),
+                                                         Ld::lone(run[j + 2 * lanes]), Ld::lone(run[j + 3 * lanes])};
+                            acc.add_vec(e, 0);
+                        }
+                    }
+#pragma unroll 4
+                    for (; j < len; j += lanes) acc.add(Ld::lone(run[j]), j);
+                    const Part p = group_combine<T>(acc.part(), gl);
+                    if (t == 0 && len > 0) store_segment<T>(p, s0 + i, a.out, a.argidx, a.aux);
+                }
+                __syncwarp();
+                continue;
+            }
+        }
+        load(q + nwarp, nb, ne);
+        if (mine && (rb > re || rb < 0)) atomicOr(a.ws.err, kErrInvalid);
+        const int64_t b = sg.clamp(rb), len = mine ? sg.clamp(re) - b : 0;
+        if (mine && len == 0) T::store_empty(a.out, s0 + lane, false, a.argidx, a.aux);
+        unsigned big = __ballot_sync(kAll, len > sp.most);
+        if (big) {
+            const unsigned n = big >> lane & 1u ? (unsigned)((len + sp.chunk - 1) / sp.chunk) : 0u;
+            const unsigned first = n ? atomicAdd(a.ws.task_count, n) : 0u;
+            for (; big; big &= big - 1) {
+                const int i = __ffs(big) - 1;
+                const unsigned f = __shfl_sync(kAll, first, i), c = __shfl_sync(kAll, n, i);
+                // (malformed offsets may list more: those segments stay unset)
+                for (unsigned k = lane; k < c && f + k < a.tasks; k += 32) a.ws.tasks[f + k] = SegTask{s0 + i, f, 0u};
+            }
+        }
+        warp_segments<T>(x, a.shift, sg.P0, sg.P1, s0, b, len > 0 && len <= sp.most ? (int)len : 0, gl, a.out, a.argidx,
+                         a.aux);
+    }
+}
+
+// 2. The long segments: tasks claimed from a counter by warps, which wait for
+// nobody: the next claim, then the next task's record, then its offsets load
+// while a task's elements travel.  A segment's partials go by task index;
+// the warp that stores the last one of 64 neighbours combines them, and the
+// one that finishes the last 64 combines those, in order both times.
+constexpr unsigned kTaskGroup = 64;
+
+template <class T>
+__global__ void __launch_bounds__(kGroupBlock) k_seg_long(SegGroupArgs a) {
+    using Part = typename T::Part;
+    constexpr unsigned kAll = 0xffffffffu;
+    const auto* x = static_cast<const typename T::Ld::In*>(a.x);
+    const Segs sg = seg_bounds(a.off, a.nseg);
+    const SegSplit sp = seg_split_lengths(sg.P1 - sg.P0, a.nseg, a.tasks);
+    const int lane = threadIdx.x & 31;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // k_seg_group is done and its list visible
+    const unsigned listed = __ldcg(a.ws.task_count);
+    const unsigned ntask = listed < a.tasks ? listed : a.tasks;
+    Part* parts = reinterpret_cast<Part*>(a.ws.head);
+    auto claim = [&]() { return lane == 0 ? atomicAdd(a.ws.chunk_ctr, 1u) : 0u; };
+    auto record = [&](unsigned k, int64_t& s, unsigned& first) {
+        s = k < ntask ? __ldcg(reinterpret_cast<const long long*>(&a.ws.tasks[k].seg)) : 0;
+        first = k < ntask ? __ldcg(&a.ws.tasks[k].first) : 0u;
+    };
+    if (ntask) {
+        unsigned k = __shfl_sync(kAll, claim(), 0), first;
+        int64_t s;
+        record(k, s, first);
+        int64_t b = sg.begin(s), e = sg.end(s);
+        unsigned k1 = claim();
+        while (k < ntask) {
+            k1 = __shfl_sync(kAll, k1, 0);
+            const unsigned k2 = claim();
+            int64_t s1;
+            unsigned first1;
+            record(k1, s1, first1);
+            const unsigned c = k - first;                    // this chunk of the segment
+            const int64_t len = e - b, c0 = (int64_t)c * sp.chunk, left = len - c0;
+            const unsigned chunks = (unsigned)((len + sp.chunk - 1) / sp.chunk);
+            Part p = group_part<T, 4>(x, b + c0, (int)(left < sp.chunk ? left : sp.chunk), a.shift, sg.P0, sg.P1, lane,
+                                      32, c0);
+            const int64_t b1 = sg.begin(s1), e1 = sg.end(s1);
+            p = T::warp_reduce(p);
+            if (chunks == 1) {
+                if (lane == 0) store_segment<T>(p, s, a.out, a.argidx, a.aux);
+            } else {
+                // c's group of chunks [g0, g0 + n), counted in its first task
+                const unsigned g0 = c / kTaskGroup * kTaskGroup;
+                const unsigned n = chunks - g0 < kTaskGroup ? chunks - g0 : kTaskGroup;
+                unsigned done = 0u;
+                if (lane == 0) {
+                    parts[k] = p;
+                    __threadfence();
+                    done = atomicAdd(&a.ws.tasks[first + g0].finished, 1u) == n - 1;
+                }
+                if (__shfl_sync(kAll, done, 0)) {
+                    __threadfence();
+                    auto gather = [&](unsigned from, unsigned count, unsigned step) {
+                        Part q = T::part_init();
+                        for (unsigned i = lane; i < count && from + i * step < a.tasks; i += 32)
+                            q = T::combine(q, ld_cg_any(parts + from + i * step));
+                        return T::warp_reduce(q);
+                    };
+                    Part q = gather(first + g0, n, 1);
+                    const unsigned groups = (chunks + kTaskGroup - 1) / kTaskGroup;
+                    bool last = groups == 1;
+                    if (!last) {
+                        // the groups of a segment are counted in its second task
+                        done = 0u;
+                        if (lane == 0) {
+                            parts[first + g0] = q;
+                            __threadfence();
+                            done = atomicAdd(&a.ws.tasks[first + 1].finished, 1u) == groups - 1;
+                        }
+                        last = __shfl_sync(kAll, done, 0) != 0u;
+                        if (last) {
+                            __threadfence();
+                            q = gather(first, groups, kTaskGroup);
+                        }
+                    }
+                    if (last && lane == 0) store_segment<T>(q, s, a.out, a.argidx, a.aux);
+                }
+            }
+            k = k1;
+            k1 = k2;
+            s = s1;
+            first = first1;
+            b = b1;
+            e = e1;
+        }
+    }
+    // The last block out clears the counters for the next launch.
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(a.ws.blk_done, 1u) == gridDim.x - 1) {
+            *a.ws.chunk_ctr = 0u;
+            *a.ws.task_count = 0u;
             *a.ws.blk_done = 0u;
         }
     }

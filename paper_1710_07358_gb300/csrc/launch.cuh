@@ -18,6 +18,30 @@ cudaError_t launch_segmented(const SegArgs& a, int grid, int block, cudaStream_t
     return cudaGetLastError();
 }
 
+template <class T>
+cudaError_t launch_seg_group(const SegGroupArgs& a, int grid, int block, cudaStream_t st) {
+    k_seg_group<T><<<grid, block, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+// Launched as a programmatic dependent of k_seg_group, always the launch
+// before it: its blocks take their places as that one's leave, and wait for
+// its end (griddepcontrol.wait) before they read the list it made.
+template <class T>
+cudaError_t launch_seg_long(const SegGroupArgs& a, int grid, int block, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_seg_long<T>, a);
+    return cudaGetLastError();
+}
+
 template <class T, int U, int VB>
 cudaError_t launch_rows(const RowArgs& a, int grid, int block, cudaStream_t st) {
     k_rows<T, U, VB><<<grid, block, 0, st>>>(a);
@@ -108,6 +132,12 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
                 KernelEntry{reinterpret_cast<const void*>(&k_axis_finish<T>),
                             reinterpret_cast<void*>(&launch_axis_finish<T>)});
         reg_add(KernelKey{K_AXIS_EMPTY, dtype, op, prec, aux, 0, 0},
+        KernelEntry sg{reinterpret_cast<const void*>(&k_seg_group<T>), reinterpret_cast<void*>(&launch_seg_group<T>)};
+        sg.part_bytes = (int)sizeof(typename T::Part);
+        reg_add(KernelKey{K_SEG_GROUP, dtype, op, prec, aux, 0, 0}, sg);
+        reg_add(KernelKey{K_SEG_LONG, dtype, op, prec, aux, 0, 0},
+                KernelEntry{reinterpret_cast<const void*>(&k_seg_long<T>),
+                            reinterpret_cast<void*>(&launch_seg_long<T>)});
                 KernelEntry{reinterpret_cast<const void*>(&k_axis_empty<T>),
                             reinterpret_cast<void*>(&launch_axis_empty<T>)});
     }

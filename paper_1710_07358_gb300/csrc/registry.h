@@ -12,6 +12,7 @@ struct ReduceArgs;
 struct SegArgs;
 struct RowArgs;
 struct RowGroupArgs;
+struct SegGroupArgs;
 struct AxisArgs;
 struct AxisBwdArgs;
 struct ScanArgs;
@@ -21,7 +22,9 @@ enum Kind : uint8_t {
     K_REDUCE = 0, K_SEGMENTED = 1, K_BACKWARD = 2, K_COMBINE = 3, K_ROWS = 4,
     K_AXIS = 5, K_AXIS_FINISH = 6, K_AXIS_EMPTY = 7, K_AXIS_BACKWARD = 8, K_SCAN = 9,
     K_REDUCE_TAIL = 10, // k_reduce with claimed tail tiles (large inputs)
-    K_ROWS_GROUP = 11   // a group of lanes per row (short rows, any alignment)
+    K_ROWS_GROUP = 11,  // a group of lanes per row (short rows, any alignment)
+    K_SEG_GROUP = 12,   // many segments: the short ones,
+    K_SEG_LONG = 13     // and the long ones
 };
 enum Aux : uint8_t { AUX_NONE = 0, AUX_ARG = 1, AUX_PROD = 2 };
 
@@ -33,6 +36,7 @@ struct KernelKey {
 using ReduceLaunch = cudaError_t (*)(const ReduceArgs&, int grid, int block, cudaStream_t);
 using SegLaunch = cudaError_t (*)(const SegArgs&, int grid, int block, cudaStream_t);
 using RowLaunch = cudaError_t (*)(const RowArgs&, int grid, int block, cudaStream_t);
+using SegGroupLaunch = cudaError_t (*)(const SegGroupArgs&, int grid, int block, cudaStream_t);
 using RowGroupLaunch = cudaError_t (*)(const RowGroupArgs&, int grid, int block, cudaStream_t);
 using AxisLaunch = cudaError_t (*)(const AxisArgs&, int grid, int block, cudaStream_t);
 using AxisBwdLaunch = cudaError_t (*)(const AxisBwdArgs&, int grid, int block, cudaStream_t);
@@ -43,7 +47,7 @@ using CombineLaunch = cudaError_t (*)(const char* parts, int count, void* out, i
 struct KernelEntry {
     const void* fn;      // the __global__ function (occupancy queries)
     void* launch;        // one of the *Launch types above, by kind
-    int part_bytes = 0;  // K_AXIS: bytes of one cross-warp partial
+    int part_bytes = 0;  // K_AXIS, K_SEG_GROUP: bytes of one partial
     int tile_slots = 0;  // K_REDUCE_TAIL: claimed tiles a block holds partials for
     int tile_loads = 0;  // K_REDUCE_TAIL: vectors a thread loads per round of a tile
 };

@@ -1,7 +1,8 @@
 // Combiner traits.  A trait describes one (element type, combiner, precision)
 // of the reduction x_0 (x) ... (x) x_{n-1} (Section 1.1):
 //
-//   Ld        element loader: storage type In, compute type E, vector decode
+//   Ld        element loader: storage type In, compute type E, vector decode,
+//             one element from memory (one) or from its stored value (lone)
 //   Acc       per-thread accumulator (the "private variable" of Section 2.3)
 //   Part      value exchanged between threads and blocks
 //   init / add / add_vec    identity and accumulation of elements
@@ -35,6 +36,7 @@ struct LdF32 {
         for (int k = 0; k < VB / 4; k++) e[k] = __uint_as_float(w.w[k]);
     }
     __device__ __forceinline__ static E one(const In* x, int64_t i) { return __ldg(x + i); }
+    __device__ __forceinline__ static E lone(In v) { return v; }
 };
 
 // bfloat16 is the high half of a binary32: widening is a shift.
@@ -51,8 +53,9 @@ struct LdBF16 {
         }
     }
     __device__ __forceinline__ static E one(const In* x, int64_t i) {
-        return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short*>(x) + i) << 16);
+        return lone(__ldg(reinterpret_cast<const unsigned short*>(x) + i));
     }
+    __device__ __forceinline__ static E lone(In v) { return __uint_as_float((uint32_t)v << 16); }
 };
 
 struct LdF16 {
@@ -71,8 +74,9 @@ struct LdF16 {
         }
     }
     __device__ __forceinline__ static E one(const In* x, int64_t i) {
-        return __half2float(__ushort_as_half(__ldg(reinterpret_cast<const unsigned short*>(x) + i)));
+        return lone(__ldg(reinterpret_cast<const unsigned short*>(x) + i));
     }
+    __device__ __forceinline__ static E lone(In v) { return __half2float(__ushort_as_half(v)); }
 };
 
 struct LdF64 {
@@ -85,6 +89,7 @@ struct LdF64 {
         for (int k = 0; k < VB / 8; k++) e[k] = __hiloint2double((int)w.w[2 * k + 1], (int)w.w[2 * k]);
     }
     __device__ __forceinline__ static E one(const In* x, int64_t i) { return __ldg(x + i); }
+    __device__ __forceinline__ static E lone(In v) { return v; }
 };
 
 struct LdI32 {
@@ -97,6 +102,7 @@ struct LdI32 {
         for (int k = 0; k < VB / 4; k++) e[k] = (int32_t)w.w[k];
     }
     __device__ __forceinline__ static E one(const In* x, int64_t i) { return __ldg(x + i); }
+    __device__ __forceinline__ static E lone(In v) { return v; }
 };
 
 struct LdU32 {
@@ -109,6 +115,7 @@ struct LdU32 {
         for (int k = 0; k < VB / 4; k++) e[k] = w.w[k];
     }
     __device__ __forceinline__ static E one(const In* x, int64_t i) { return __ldg(x + i); }
+    __device__ __forceinline__ static E lone(In v) { return v; }
 };
 
 // int64 is handled as uint64 bit patterns (two's-complement wrap-around).
@@ -124,6 +131,7 @@ struct LdI64 {
     __device__ __forceinline__ static E one(const In* x, int64_t i) {
         return (uint64_t)__ldg(reinterpret_cast<const long long*>(x) + i);
     }
+    __device__ __forceinline__ static E lone(In v) { return (uint64_t)v; }
 };
 
 // Output writers for float-valued results.
