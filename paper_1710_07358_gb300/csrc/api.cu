@@ -1006,6 +1006,8 @@ static pr_status segmented_common(const void* x, const int64_t* offsets, int64_t
     if ((s = check_aligned(x, dtype, "x")) != PR_OK) return s;
     const int auxk = argidx ? AUX_ARG : (aux ? AUX_PROD : AUX_NONE);
     ensure_registered();
+    if (offsets && nseg >= (auxk == AUX_NONE ? kSegGroupMin : kSegGroupMinHeavy))
+        return run_seg_group(x, offsets, nseg, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream);
     const pr_config c = lookup_cfg(PR_KIND_SEGMENTED, dtype, op, precision, nseg);
     return run_segmented(x, offsets, cols, nseg, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream, c);
 }
@@ -1039,8 +1041,6 @@ pr_status pr_reduce_rows(const void* x, int64_t rows, int64_t cols, pr_dtype dty
         const int auxk = argidx ? AUX_ARG : (aux ? AUX_PROD : AUX_NONE);
         pr_status s = run_rows_group(x, rows, cols, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream);
         if (s != PR_ERR_UNSUPPORTED) return s;
-    if (offsets && nseg >= (auxk == AUX_NONE ? kSegGroupMin : kSegGroupMinHeavy))
-        return run_seg_group(x, offsets, nseg, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream);
         const pr_config c = lookup_cfg(PR_KIND_ROWS, dtype, op, precision, rows * cols);
         s = run_rows(x, rows, cols, dtype, op, precision, auxk, out, argidx, aux, (cudaStream_t)stream, c);
         if (s != PR_ERR_UNSUPPORTED) return s;

@@ -122,6 +122,12 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
         reg_add(KernelKey{K_ROWS_GROUP, dtype, op, prec, aux, 0, 0},
                 KernelEntry{reinterpret_cast<const void*>(&k_rows_group<T>),
                             reinterpret_cast<void*>(&launch_rows_group<T>)});
+        KernelEntry sg{reinterpret_cast<const void*>(&k_seg_group<T>), reinterpret_cast<void*>(&launch_seg_group<T>)};
+        sg.part_bytes = (int)sizeof(typename T::Part);
+        reg_add(KernelKey{K_SEG_GROUP, dtype, op, prec, aux, 0, 0}, sg);
+        reg_add(KernelKey{K_SEG_LONG, dtype, op, prec, aux, 0, 0},
+                KernelEntry{reinterpret_cast<const void*>(&k_seg_long<T>),
+                            reinterpret_cast<void*>(&launch_seg_long<T>)});
         reg_axis<T, 2, 0>(dtype, op, prec, aux);
         reg_axis<T, 2, 16>(dtype, op, prec, aux);
         reg_axis<T, 2, 32>(dtype, op, prec, aux);
@@ -132,12 +138,6 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
                 KernelEntry{reinterpret_cast<const void*>(&k_axis_finish<T>),
                             reinterpret_cast<void*>(&launch_axis_finish<T>)});
         reg_add(KernelKey{K_AXIS_EMPTY, dtype, op, prec, aux, 0, 0},
-        KernelEntry sg{reinterpret_cast<const void*>(&k_seg_group<T>), reinterpret_cast<void*>(&launch_seg_group<T>)};
-        sg.part_bytes = (int)sizeof(typename T::Part);
-        reg_add(KernelKey{K_SEG_GROUP, dtype, op, prec, aux, 0, 0}, sg);
-        reg_add(KernelKey{K_SEG_LONG, dtype, op, prec, aux, 0, 0},
-                KernelEntry{reinterpret_cast<const void*>(&k_seg_long<T>),
-                            reinterpret_cast<void*>(&launch_seg_long<T>)});
                 KernelEntry{reinterpret_cast<const void*>(&k_axis_empty<T>),
                             reinterpret_cast<void*>(&launch_axis_empty<T>)});
     }
