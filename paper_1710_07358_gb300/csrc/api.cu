@@ -710,9 +710,40 @@ static pr_status axis_scratch(cudaStream_t st, size_t bytes, char** out) {
     return PR_OK;
 }
 
+// Row splits of `tiles` blocks' worth of work with `resident` blocks at once:
+// the least estimated time.  The input streams in stream_us when the waves of
+// blocks are full (a single wave streams at full rate from about 0.6 of the
+// GPU on); SMs that finish early cost about 0.08 of a wave ([16, 4096, 4096]
+// fp32 sum: 173 us in one wave, 160 in many); a wave about 2 us to start and
+// to combine, a finishing pass as much; the partials `part` of the input's
+// traffic per split.
+static int64_t axis_splits(int64_t tiles, int64_t resident, int64_t most, double stream_us, double part) {
+    int64_t best = 1;
+    double least = 1e30;
+    for (int64_t s = 1; s <= most && s <= 1024; s++) {
+        const double w = (double)tiles * s / (double)resident, waves = std::ceil(w);
+        const double fill = w <= 1.0 ? (0.6 / w > 1.0 ? 0.6 / w : 1.0) : waves / w;
+        const double us = stream_us * (fill + 0.08 / waves + (s > 1 ? part * s : 0.0)) + 2.0 * waves + (s > 1 ? 2.0 : 0.0);
+        if (us < least) {
+            least = us;
+            best = s;
+        }
+        if (waves > 16.0) break;
+    }
+    return best;
+}
+
 // Reduction of the middle axis of [outer, n, inner] (inner > 1, outer > 0).
-// The launch: warps per (slab, column group) times row splits, enough warps
-// for about two waves of the resident ones; splits > 1 add a finishing pass.
+// The launch: a warp per (slab, column group), times row splits where those do
+// not fill the GPU twice.  Splits of a warp each leave a partial each; where
+// those come to more than a twentieth of the input's traffic, the warps of a
+// block share a split instead, and axis_splits has their number (measured on
+// GB300, us: [64, 577, 768] fp32 maximum with index 77 with 49 splits of a
+// warp, 33 shared; [4096, 16, 512] sum 44 and 29; [16, 4096, 4096] sum 159 and
+// 166, maximum 168 and 199).  Inputs below 7 MB are bound by latency either
+// way, and columns that are not whole vectors keep more rows in flight in the
+// smaller kernel ([1, 5000, 4099] maximum 49 and 57).  splits > 1 add a
+// finishing pass.
 static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner, int dtype, int op, int prec,
                           int aux, void* out, int64_t* argidx, pr_prod_aux* paux, cudaStream_t st,
                           const pr_config& cfg) {
@@ -720,7 +751,7 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
     DevInfo di;
     pr_status s = device_info(&di, nullptr);
     if (s != PR_OK) return s;
-    AxisArgs a{x, outer, n, inner, 0, 1, 0, 1, 0, out, argidx, paux, 0, nullptr};
+    AxisArgs a{x, outer, n, inner, 0, 1, 0, 1, 1, 0, out, argidx, paux, 0, nullptr};
     if (n == 0) {
         const KernelEntry* e = reg_find(KernelKey{K_AXIS_EMPTY, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec,
                                                   (uint8_t)aux, 0, 0});
@@ -738,7 +769,7 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
     const KernelEntry* e = reg_find(KernelKey{K_AXIS, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux,
                                               (uint8_t)cfg.unroll, (uint8_t)vb});
     if (!e) return fail(PR_ERR_UNSUPPORTED, "no axis kernel for dtype %d op %d precision %d", dtype, op, prec);
-    const pr_config c = fit_block(e, cfg);
+    pr_config c = fit_block(e, cfg);
     int occ = 0;
     s = occupancy(e->fn, c.block, &occ);
     if (s != PR_OK) return s;
@@ -752,26 +783,46 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
     a.groups = (a.qv + bx - 1) / bx;
     const int64_t tiles = outer * a.groups;
     const int64_t want = (int64_t)di.sms * bps * (c.block / 32) * 2;   // two waves of resident warps
-    const int64_t ry = 32 / bx;
-    int64_t max_split = n / (ry * c.unroll * 4);                        // >= 4 unrolled steps per warp
-    if (max_split < 1) max_split = 1;
-    if (max_split > 1024) max_split = 1024;
-    int64_t splits = (want + tiles - 1) / tiles;
+    const int64_t step = 32 / bx * c.unroll;                           // rows of a warp's unrolled step
+    const int64_t max_split = n / (step * 4) > 1 ? n / (step * 4) : 1; // >= 4 steps per warp
+    const double stream_us = (double)outer * n * inner * es / 6.8e6;
+    const double part = 2.0 * e->part_bytes / ((double)n * es);        // partials' traffic per split, of the input's
+    int64_t splits = (want + tiles - 1) / tiles;                       // a warp each
     if (splits > max_split) splits = max_split;
-    if (splits < 1) splits = 1;
-    // a split holds fewer than 2^31 rows (the float arg-extremum keeps its
-    // row as a 32-bit offset within the split)
+    if (splits > 1024) splits = 1024;
+    if (splits > 1 && vb == 32 && stream_us > 1.0 && part * splits > 0.05) {
+        // the warps of a block share a tile's rows, then blocks split them
+        const KernelEntry* ec = reg_find(KernelKey{K_AXIS_COOP, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux, 2, 32});
+        if (!ec) return fail(PR_ERR_UNSUPPORTED, "no axis kernel for dtype %d op %d precision %d", dtype, op, prec);
+        e = ec;
+        const int64_t most = n / (32 / bx * 2 * 4) > 1 ? n / (32 / bx * 2 * 4) : 1;
+        while (a.coop < kAxisCoop && 2 * a.coop <= most) a.coop *= 2;
+        c.block = 32 * a.coop;
+        s = occupancy(e->fn, c.block, &occ);
+        if (s != PR_OK) return s;
+        if (occ < 1) return fail(PR_ERR_UNSUPPORTED, "axis kernel cannot run with %d threads per block", c.block);
+        splits = axis_splits(tiles, (int64_t)di.sms * occ, most / a.coop, stream_us, part);
+    }
+    a.splits = splits;
+    // a warp holds fewer than 2^31 rows (the float arg-extremum keeps its
+    // row as a 32-bit offset from the warp's first one)
     const int64_t kMaxSplitRows = (int64_t)1 << 30;
-    if ((n + splits - 1) / splits > kMaxSplitRows) splits = (n + kMaxSplitRows - 1) / kMaxSplitRows;
-    a.rows_per_split = (n + splits - 1) / splits;
-    a.splits = (n + a.rows_per_split - 1) / a.rows_per_split;
+    if ((n + a.splits * a.coop - 1) / (a.splits * a.coop) > kMaxSplitRows)
+        a.splits = (n + kMaxSplitRows * a.coop - 1) / (kMaxSplitRows * a.coop);
+    a.rows_per_split = (n + a.splits * a.coop - 1) / (a.splits * a.coop);
+    // (splits past the last row would leave partials of no rows: identities)
+    a.splits = (n + a.rows_per_split * a.coop - 1) / (a.rows_per_split * a.coop);
+    // the scratch's growth, the two launches and what they leave in it belong
+    // together, whatever other host threads enqueue on the stream
+    std::unique_lock<std::mutex> pair(g_pair_mu, std::defer_lock);
     if (a.splits > 1) {
+        pair.lock();
         char* sc = nullptr;
         s = axis_scratch(st, (size_t)(outer * inner) * (size_t)a.splits * (size_t)e->part_bytes, &sc);
         if (s != PR_OK) return s;
         a.scratch = sc;
     }
-    const int64_t warps = tiles * a.splits;
+    const int64_t warps = tiles * a.splits * a.coop;
     const int wpb = c.block / 32;
     const int64_t grid = (warps + wpb - 1) / wpb;
     if (grid > 0x7fffffff) return fail(PR_ERR_INVALID, "axis reduction too large for one launch");
@@ -886,6 +937,29 @@ static pr_status run_axis_backward(int op, int dtype, const void* x, int64_t out
     if (!e) return fail(PR_ERR_UNSUPPORTED, "no axis backward kernel for dtype %d", dtype);
     const int ve = vb ? vb / es : 1;
     AxisBwdArgs a{x, g, argidx, aux, gi, outer, n, inner, inner / ve, op};
+    // by columns where the lanes fit the row: three of four have a column, or
+    // all for the fp64 product, which is bound by its divisions
+    int bx = 1;
+    while (bx < 32 && bx < a.qv) bx <<= 1;
+    const int64_t groups = (a.qv + bx - 1) / bx;
+    const bool divides = op == PR_PROD && dtype == PR_F64;
+    if (divides ? a.qv == groups * bx : a.qv * 4 >= groups * bx * 3) {
+        // steps of 32 / bx rows: up to 16 a warp (a column's state is loaded
+        // once a warp) while 64 warps an SM are left, more where the warps
+        // fill the GPU eight times over; with one step a warp there is
+        // nothing to hold
+        const int64_t steps = (n + 32 / bx - 1) / (32 / bx);
+        const int64_t full = (int64_t)di.sms * 64;
+        int64_t per = outer * groups * steps / full;
+        per = per > 16 * 8 ? per / 8 : (per > 16 ? 16 : (per < 1 ? 1 : per));
+        const int64_t splits = (steps + per - 1) / per;
+        if (per > 1 && (outer * groups * splits + 7) / 8 <= 0x7fffffff) {
+            PR_INJECT_LAUNCH();
+            cudaError_t err = launch_axis_backward_cols(a, dtype == PR_F64, vb, bx, groups, splits, st);
+            if (err != cudaSuccess) return fail(PR_ERR_CUDA, "axis backward launch: %s", cudaGetErrorString(err));
+            return PR_OK;
+        }
+    }
     const int64_t total = outer * n * a.qv;
     int64_t grid = (total + 255) / 256;
     const int64_t cap = (int64_t)di.sms * 64;

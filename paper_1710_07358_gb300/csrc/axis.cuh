@@ -11,8 +11,14 @@
 //   load instruction still touches 32 neighbouring vectors.  Each lane issues
 //   U rows' loads before accumulating any of them.  The lanes that share a
 //   column then combine by an xor butterfly over the row bits of the lane
-//   index, in a fixed order.  With one split the warp writes the outputs; with
-//   more, it writes its partials, and k_axis_finish combines each output's
+//   index, in a fixed order.  Where tiles alone leave warps idle, the warps of
+//   a block share a tile's rows first and combine through shared memory (in
+//   warp order), and only then are the rows split over blocks: a partial per
+//   warp and output cost more traffic than the input where the axis is short
+//   ([64, 577, 768] fp32 maximum with index: 49 splits wrote and read 38 MB
+//   each of 16-byte partials for 113 MB of input; with shared splits 77 -> 33
+//   us, 0.51 of a 6.8 TB/s copy: one wave of blocks, bound by latency).  With one split the outputs
+//   are written; with more, the partials, and k_axis_finish combines each output's
 //   partials in a fixed order (one thread per output folding the splits in
 //   order, or with many splits one warp per output and a fixed tree), so
 //   results are deterministic for a fixed launch shape.
@@ -29,8 +35,9 @@ struct AxisArgs {
     int64_t qv;               // column vectors per row: inner / VE
     int bx;                   // lanes per row (power of two, <= 32)
     int64_t groups;           // column groups per row: ceil(qv / bx)
-    int64_t splits;           // row splits
-    int64_t rows_per_split;
+    int64_t splits;           // row splits that leave a partial each (one warp's, or a block's)
+    int coop;                 // warps of a block that share a split (k_axis COOP; else 1)
+    int64_t rows_per_split;   // rows of one warp
     void* out;
     int64_t* argidx;
     pr_prod_aux* aux;
@@ -42,6 +49,8 @@ struct AxisArgs {
 // Up to this many splits the finishing pass takes one thread per output
 // (coalesced over outputs); beyond it, one warp per output.
 constexpr int kAxisThreadFinish = 64;
+// Most warps of a block that share a split (their partials meet in shared memory).
+constexpr int kAxisCoop = 8;
 
 // A column's elements reach its accumulator in increasing index order, so a
 // trait may take them with a cheaper in-order step (add_ordered).
@@ -63,6 +72,15 @@ __device__ __forceinline__ void add_in_order(typename T::Acc& a, typename T::Ld:
     else T::add(a, v, i);
 }
 
+// Column elements (a divisor of VE) whose partials of kAxisCoop warps meet in
+// shared memory at a time: up to 16 KB.
+template <class T, int VE>
+struct AxisPhase {
+    static constexpr int kBytes = kAxisCoop * 32 * (int)sizeof(typename T::Part);
+    static constexpr int fit(int k) { return k > 1 && k * kBytes > 16384 ? fit(k / 2) : k; }
+    static constexpr int value = fit(VE);
+};
+
 template <int VB, class Ld>
 __device__ __forceinline__ void axis_load(const typename Ld::In* x, int64_t e0, typename Ld::E (&e)[VB ? VB / Ld::ES : 1]) {
     if constexpr (VB == 0) {
@@ -73,8 +91,12 @@ __device__ __forceinline__ void axis_load(const typename Ld::In* x, int64_t e0, 
     }
 }
 
-template <class T, int U, int VB>
-__global__ void __launch_bounds__(MaxBlock<T>::value) k_axis(AxisArgs a) {
+// COOP: the variant whose blocks' warps share a split (a.coop of them, the
+// whole block).  It is compiled apart because its shared memory and registers
+// cost the other resident warps ([4096, 16, 512] fp64 minimum with index 79 us
+// without it in the kernel, 91 with).
+template <class T, int U, int VB, bool COOP>
+__global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_axis(AxisArgs a) {
     using Ld = typename T::Ld;
     using In = typename Ld::In;
     using E = typename Ld::E;
@@ -84,23 +106,32 @@ __global__ void __launch_bounds__(MaxBlock<T>::value) k_axis(AxisArgs a) {
     using G = typename GR::Part;
     constexpr int VE = VB ? VB / Ld::ES : 1;
     const In* x = static_cast<const In*>(a.x);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // k_axis_finish waits for this grid's end
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t tiles = a.outer * a.groups;
-    if (wid >= tiles * a.splits) return;  // whole warps (blockDim is a multiple of 32)
-    const int64_t tile = wid / a.splits, s = wid - tile * a.splits;
+    const int64_t wsplits = a.splits * a.coop;                   // warps per tile
+    if (wid >= tiles * wsplits) return;  // whole warps (blockDim is a multiple of 32); none where warps share a split
+    const int64_t tile = wid / wsplits, ws = wid - tile * wsplits;
+    const int64_t s = ws / a.coop;
     const int64_t p = tile / a.groups, grp = tile - p * a.groups;
     const int bx = a.bx, ry = 32 / bx;
     const int tx = lane & (bx - 1), ty = lane / bx;
     const int64_t col = grp * bx + tx;
     const bool has = col < a.qv;
-    const int64_t r0 = s * a.rows_per_split;
+    const int64_t r0 = ws * a.rows_per_split;
     const int64_t r1 = r0 + a.rows_per_split < a.n ? r0 + a.rows_per_split : a.n;
     const int64_t slab = p * a.n * a.inner + col * VE;  // element offset of (p, row 0, this column)
 
     Acc acc[VE];
+    constexpr bool kBlocked = COOP && !Exact<T>::value && sizeof(Acc) == 4 && VE * sizeof(Part) <= 64;   // (registers)
+    constexpr int kBlockSteps = sizeof(Part) == 8 ? 8 : 4;   // (fp64 additions are slow)
+    Part total[kBlocked ? VE : 1];
 #pragma unroll
-    for (int k = 0; k < VE; k++) acc[k] = T::init();
+    for (int k = 0; k < VE; k++) {
+        acc[k] = T::init();
+        if constexpr (kBlocked) total[k] = T::part_init();
+    }
     if constexpr (HasOrderedPair<T>::value) {
         // per element the running extremum and its row relative to r0 (a
         // split holds fewer than 2^31 rows): three operations an element
@@ -152,6 +183,27 @@ __global__ void __launch_bounds__(MaxBlock<T>::value) k_axis(AxisArgs a) {
         }
     } else if (has) {
         int64_t r = r0 + ty;
+        // an inexact 32-bit accumulator joins its Part every kBlockSteps
+        // steps: a shorter chain of roundings, whatever the split
+        if constexpr (kBlocked) {
+            for (; r + (int64_t)(kBlockSteps * U - 1) * ry < r1;) {
+#pragma unroll 1
+                for (int b = 0; b < kBlockSteps; b++, r += (int64_t)U * ry) {
+                    E e[U][VE];
+#pragma unroll
+                    for (int u = 0; u < U; u++) axis_load<VB, Ld>(x, slab + (r + (int64_t)u * ry) * a.inner, e[u]);
+#pragma unroll
+                    for (int u = 0; u < U; u++)
+#pragma unroll
+                        for (int k = 0; k < VE; k++) add_in_order<T>(acc[k], e[u][k], r + (int64_t)u * ry);
+                }
+#pragma unroll
+                for (int k = 0; k < VE; k++) {
+                    total[k] = T::combine(total[k], T::to_part(acc[k]));
+                    acc[k] = T::init();
+                }
+            }
+        }
         for (; r + (int64_t)(U - 1) * ry < r1; r += (int64_t)U * ry) {
             E e[U][VE];
 #pragma unroll
@@ -169,20 +221,47 @@ __global__ void __launch_bounds__(MaxBlock<T>::value) k_axis(AxisArgs a) {
         }
     }
     const bool f64 = a.out_f64 != 0;
+    auto result = [&](int k, const Part& q) {
+        if (ty != 0 || !has) return;
+        const int64_t o = p * a.inner + col * VE + k;
+        const G g = GR::up(q);
+        if (a.splits == 1) {
+            GR::store(a.out, o, g, f64);
+            GR::store_aux(a.argidx, a.aux, o, g, 0);
+        } else {
+            const int64_t nout = a.outer * a.inner;
+            reinterpret_cast<G*>(a.scratch)[a.splits <= kAxisThreadFinish ? s * nout + o : o * a.splits + s] = g;
+        }
+    };
+    // a warp's column elements combine across its rows' lanes; then (COOP),
+    // KP elements at a time, across the block's warps in warp order, each
+    // element by one of the warps
+    if constexpr (COOP) {
+        constexpr int KP = AxisPhase<T, VE>::value;
+        __shared__ Part s_part[KP][kAxisCoop][32];
+        const int warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < VE; k++) {
-        Part q = T::to_part(acc[k]);
-        for (int m = 16; m >= bx; m >>= 1) q = T::combine(q, shfl_xor_any(q, m));
-        if (ty == 0 && has) {
-            const int64_t o = p * a.inner + col * VE + k;
-            const G g = GR::up(q);
-            if (a.splits == 1) {
-                GR::store(a.out, o, g, f64);
-                GR::store_aux(a.argidx, a.aux, o, g, 0);
-            } else {
-                const int64_t nout = a.outer * a.inner;
-                reinterpret_cast<G*>(a.scratch)[a.splits <= kAxisThreadFinish ? s * nout + o : o * a.splits + s] = g;
+        for (int k = 0; k < VE; k++) {
+            Part q = T::to_part(acc[k]);
+            if constexpr (kBlocked) q = T::combine(total[k], q);
+            for (int m = 16; m >= bx; m >>= 1) q = T::combine(q, shfl_xor_any(q, m));
+            s_part[k % KP][warp][lane] = q;
+            if (k % KP == KP - 1) {
+                __syncthreads();
+                for (int j = warp; j < KP; j += a.coop) {
+                    q = s_part[j][0][lane];
+                    for (int w = 1; w < a.coop; w++) q = T::combine(q, s_part[j][w][lane]);
+                    result(k - (KP - 1) + j, q);
+                }
+                if (k < VE - 1) __syncthreads();   // before the slots are written again
             }
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < VE; k++) {
+            Part q = T::to_part(acc[k]);
+            for (int m = 16; m >= bx; m >>= 1) q = T::combine(q, shfl_xor_any(q, m));
+            result(k, q);
         }
     }
 }
@@ -194,6 +273,7 @@ template <class T>
 __global__ void __launch_bounds__(256) k_axis_finish(AxisArgs a) {
     using GR = GridR<T>;
     using G = typename GR::Part;
+    asm volatile("griddepcontrol.wait;" ::: "memory");   // launched as k_axis' programmatic dependent
     const int64_t nout = a.outer * a.inner;
     const G* part = reinterpret_cast<const G*>(a.scratch);
     if (a.splits <= kAxisThreadFinish) {
@@ -224,6 +304,28 @@ __global__ void __launch_bounds__(256) k_axis_empty(AxisArgs a) {
     const int64_t nout = a.outer * a.inner;
     for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < nout; o += (int64_t)gridDim.x * blockDim.x)
         T::store_empty(a.out, o, a.out_f64 != 0, a.argidx, a.aux);
+}
+
+// One vector store of VB bytes.
+template <class F, int VB>
+__device__ __forceinline__ void st_vec(F* p, const F (&v)[VB / sizeof(F)]);
+
+template <>
+__device__ __forceinline__ void st_vec<float, 16>(float* p, const float (&v)[4]) {
+    asm volatile("st.global.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+}
+template <>
+__device__ __forceinline__ void st_vec<float, 32>(float* p, const float (&v)[8]) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
+}
+template <>
+__device__ __forceinline__ void st_vec<double, 16>(double* p, const double (&v)[2]) {
+    asm volatile("st.global.v2.f64 [%0], {%1,%2};" ::"l"(p), "d"(v[0]), "d"(v[1]) : "memory");
+}
+template <>
+__device__ __forceinline__ void st_vec<double, 32>(double* p, const double (&v)[4]) {
+    asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
 }
 
 struct AxisBwdArgs {
@@ -285,19 +387,7 @@ __global__ void __launch_bounds__(256) k_axis_backward(AxisBwdArgs a) {
         if constexpr (VB == 0) {
             gi[e0] = vals[0];
         } else {
-            F* dst = gi + e0;
-            if constexpr (sizeof(F) == 4 && VB == 16)
-                asm volatile("st.global.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(dst), "f"((float)vals[0]), "f"((float)vals[1]),
-                             "f"((float)vals[2]), "f"((float)vals[3]) : "memory");
-            else if constexpr (sizeof(F) == 4 && VB == 32)
-                asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst), "f"((float)vals[0]),
-                             "f"((float)vals[1]), "f"((float)vals[2]), "f"((float)vals[3]), "f"((float)vals[4]),
-                             "f"((float)vals[5]), "f"((float)vals[6]), "f"((float)vals[7]) : "memory");
-            else if constexpr (sizeof(F) == 8 && VB == 16)
-                asm volatile("st.global.v2.f64 [%0], {%1,%2};" ::"l"(dst), "d"((double)vals[0]), "d"((double)vals[1]) : "memory");
-            else
-                asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(dst), "d"((double)vals[0]), "d"((double)vals[1]),
-                             "d"((double)vals[2]), "d"((double)vals[3]) : "memory");
+            st_vec<F, VB>(gi + e0, vals);
         }
         // advance by the stride: columns, then rows, then slabs
         cq += dq;
@@ -307,6 +397,83 @@ __global__ void __launch_bounds__(256) k_axis_backward(AxisBwdArgs a) {
         const int64_t c2 = i >= a.n ? 1 : 0;
         i -= c2 * a.n;
         p += dp + c2;
+    }
+}
+
+// The same gradient with each column's grad_out and state held in registers:
+// a warp takes a group of column vectors of one slab (lanes as in k_axis: bx
+// per row, 32 / bx rows a step) and writes every `splits`-th step of its rows,
+// so that the warps of a slab write one moving window of neighbouring rows.
+// k_axis_backward re-reads them for every row, 96 bytes per 32 written for
+// the extrema; it keeps inputs too small for two steps a warp, and rows that
+// leave lanes without a column.  Bound by the write: fp32 maximum of [64, 577,
+// 768] 62 -> 20.7 us (0.80 of a 6.8 TB/s copy), of [16, 4096, 4096] 528 -> 146
+// (1.08), its sum 156 -> 147, product of [64, 577, 768] 170 -> 57 (0.58, with
+// x read; the divisions).
+template <class F, int VB, int OPK>
+__global__ void __launch_bounds__(256) k_axis_backward_cols(AxisBwdArgs a, int bx, int64_t groups, int64_t splits,
+                                                            int xvec) {
+    constexpr int VE = VB ? VB / (int)sizeof(F) : 1;
+    const int lane = threadIdx.x & 31, ry = 32 / bx;
+    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t tile = wid / splits, s = wid - tile * splits;
+    const int64_t p = tile / groups, col = (tile - p * groups) * bx + (lane & (bx - 1));
+    if (p >= a.outer || col >= a.qv) return;
+    const int64_t o0 = p * a.inner + col * VE;
+    const F* x = static_cast<const F*>(a.x);
+    F* gi = static_cast<F*>(a.gi);
+    int64_t i = s * ry + lane / bx;
+    // the product's factors of row r, loaded a row ahead of their use
+    F xe[VE];
+    auto load_x = [&](int64_t r) {
+        if (OPK != 2 || r >= a.n) return;
+        const int64_t e0 = (p * a.n + r) * a.inner + col * VE;
+        if constexpr (VB != 0) {
+            if (xvec) {
+                const Words<VB> w = ldv<VB>(x + e0);
+                memcpy(xe, w.w, VB);
+                return;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < VE; k++) xe[k] = __ldg(x + e0 + k);
+    };
+    load_x(i);
+    F gv[VE];
+    int64_t hot[VE];      // the row that gets gv, -1: none, -2: every row, -3: every row, divided by x
+    if constexpr (VB == 0) {
+        gv[0] = __ldg(static_cast<const F*>(a.g) + o0);
+    } else {
+        const Words<VB> w = ldv<VB>(static_cast<const F*>(a.g) + o0);
+        memcpy(gv, w.w, VB);
+    }
+#pragma unroll
+    for (int k = 0; k < VE; k++) {
+        hot[k] = -2;
+        if constexpr (OPK == 1) {
+            hot[k] = __ldg(a.argidx + o0 + k);
+        } else if constexpr (OPK == 2) {
+            const pr_prod_aux ax = a.aux[o0 + k];
+            gv[k] = (F)((double)gv[k] * ax.p_nz);
+            hot[k] = ax.zero_count == 0 ? -3 : (ax.zero_count == 1 ? ax.first_zero : -1);
+        }
+    }
+    for (; i < a.n; i += splits * ry) {
+        const int64_t e0 = (p * a.n + i) * a.inner + col * VE;
+        F vals[VE];
+        if constexpr (OPK == 2) {
+            F xc[VE];
+#pragma unroll
+            for (int k = 0; k < VE; k++) xc[k] = xe[k];
+            load_x(i + splits * ry);
+#pragma unroll
+            for (int k = 0; k < VE; k++) vals[k] = hot[k] == -3 ? gv[k] / xc[k] : (hot[k] == i ? gv[k] : (F)0);
+        } else {
+#pragma unroll
+            for (int k = 0; k < VE; k++) vals[k] = OPK == 0 || hot[k] == i ? gv[k] : (F)0;
+        }
+        if constexpr (VB == 0) gi[e0] = vals[0];
+        else st_vec<F, VB>(gi + e0, vals);
     }
 }
 

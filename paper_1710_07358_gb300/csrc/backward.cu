@@ -11,7 +11,8 @@
 // blocks in flight always write one window of neighbouring chunks and the
 // hardware hands the remaining blocks to whichever SMs finish first (no tail of
 // SMs still writing fixed shares).  Row-uniform values (grad_out, argidx, aux)
-// are re-read only when a block's row changes.
+// are re-read only when a block's row changes.  Rows of at most 32768 elements
+// take the flat form, k_backward_flat.
 #include "registry.h"
 #include "kernels.cuh"
 #include "axis.cuh"
@@ -19,27 +20,6 @@
 namespace pr {
 
 constexpr int kFlatBlock = 256;
-
-template <class F, int VB>
-__device__ __forceinline__ void st_vec(F* p, const F (&v)[VB / sizeof(F)]);
-
-template <>
-__device__ __forceinline__ void st_vec<float, 16>(float* p, const float (&v)[4]) {
-    asm volatile("st.global.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
-}
-template <>
-__device__ __forceinline__ void st_vec<float, 32>(float* p, const float (&v)[8]) {
-    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
-                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
-}
-template <>
-__device__ __forceinline__ void st_vec<double, 16>(double* p, const double (&v)[2]) {
-    asm volatile("st.global.v2.f64 [%0], {%1,%2};" ::"l"(p), "d"(v[0]), "d"(v[1]) : "memory");
-}
-template <>
-__device__ __forceinline__ void st_vec<double, 32>(double* p, const double (&v)[4]) {
-    asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
-}
 
 // Row-uniform description of the gradient: value gv at column `hot` (or at
 // every column when hot == -2), 0 elsewhere; div: gv / x[c] at every column.
@@ -272,6 +252,32 @@ static void reg_bwd(uint8_t dtype) {
 template <class F, int VB, int OPK>
 cudaError_t launch_axis_backward(const AxisBwdArgs& a, int grid, int block, cudaStream_t st) {
     k_axis_backward<F, VB, OPK><<<grid, block, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+// Column form (k_axis_backward_cols): lanes per row, column groups and row
+// splits as in its comment.
+template <class F, int VB>
+static void axis_cols_go(const AxisBwdArgs& a, int bx, int64_t groups, int64_t splits, cudaStream_t st) {
+    const int64_t grid = (a.outer * groups * splits + 7) / 8;
+    const int xvec = VB && a.op == PR_PROD && reinterpret_cast<uintptr_t>(a.x) % VB == 0 ? 1 : 0;
+    const unsigned g = (unsigned)grid;
+    if (a.op == PR_SUM) k_axis_backward_cols<F, VB, 0><<<g, 256, 0, st>>>(a, bx, groups, splits, xvec);
+    else if (a.op == PR_PROD) k_axis_backward_cols<F, VB, 2><<<g, 256, 0, st>>>(a, bx, groups, splits, xvec);
+    else k_axis_backward_cols<F, VB, 1><<<g, 256, 0, st>>>(a, bx, groups, splits, xvec);
+}
+
+cudaError_t launch_axis_backward_cols(const AxisBwdArgs& a, bool f64, int vb, int bx, int64_t groups, int64_t splits,
+                                      cudaStream_t st) {
+    if (f64) {
+        if (vb == 32) axis_cols_go<double, 32>(a, bx, groups, splits, st);
+        else if (vb == 16) axis_cols_go<double, 16>(a, bx, groups, splits, st);
+        else axis_cols_go<double, 0>(a, bx, groups, splits, st);
+    } else {
+        if (vb == 32) axis_cols_go<float, 32>(a, bx, groups, splits, st);
+        else if (vb == 16) axis_cols_go<float, 16>(a, bx, groups, splits, st);
+        else axis_cols_go<float, 0>(a, bx, groups, splits, st);
+    }
     return cudaGetLastError();
 }
 

@@ -54,15 +54,25 @@ cudaError_t launch_rows_group(const RowGroupArgs& a, int grid, int block, cudaSt
     return cudaGetLastError();
 }
 
-template <class T, int U, int VB>
+template <class T, int U, int VB, bool COOP>
 cudaError_t launch_axis(const AxisArgs& a, int grid, int block, cudaStream_t st) {
-    k_axis<T, U, VB><<<grid, block, 0, st>>>(a);
+    k_axis<T, U, VB, COOP><<<grid, block, 0, st>>>(a);
     return cudaGetLastError();
 }
 
+// A programmatic dependent of k_axis, always the launch before it.
 template <class T>
 cudaError_t launch_axis_finish(const AxisArgs& a, int grid, int block, cudaStream_t st) {
-    k_axis_finish<T><<<grid, block, 0, st>>>(a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_axis_finish<T>, a);
     return cudaGetLastError();
 }
 
@@ -101,11 +111,12 @@ void reg_one(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain, b
     }
 }
 
-template <class T, int U, int VB>
+template <class T, int U, int VB, bool COOP = false>
 void reg_axis(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux) {
-    KernelEntry e{reinterpret_cast<const void*>(&k_axis<T, U, VB>), reinterpret_cast<void*>(&launch_axis<T, U, VB>)};
+    KernelEntry e{reinterpret_cast<const void*>(&k_axis<T, U, VB, COOP>),
+                  reinterpret_cast<void*>(&launch_axis<T, U, VB, COOP>)};
     e.part_bytes = (int)sizeof(typename GridR<T>::Part);
-    reg_add(KernelKey{K_AXIS, dtype, op, prec, aux, (uint8_t)U, (uint8_t)VB}, e);
+    reg_add(KernelKey{COOP ? K_AXIS_COOP : K_AXIS, dtype, op, prec, aux, (uint8_t)U, (uint8_t)VB}, e);
 }
 
 // Register every (unroll, vector width) of one trait; plain-reduce traits
@@ -134,6 +145,7 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
         reg_axis<T, 4, 0>(dtype, op, prec, aux);
         reg_axis<T, 4, 16>(dtype, op, prec, aux);
         reg_axis<T, 4, 32>(dtype, op, prec, aux);
+        reg_axis<T, 2, 32, true>(dtype, op, prec, aux);
         reg_add(KernelKey{K_AXIS_FINISH, dtype, op, prec, aux, 0, 0},
                 KernelEntry{reinterpret_cast<const void*>(&k_axis_finish<T>),
                             reinterpret_cast<void*>(&launch_axis_finish<T>)});

@@ -24,7 +24,8 @@ enum Kind : uint8_t {
     K_REDUCE_TAIL = 10, // k_reduce with claimed tail tiles (large inputs)
     K_ROWS_GROUP = 11,  // a group of lanes per row (short rows, any alignment)
     K_SEG_GROUP = 12,   // many segments: the short ones,
-    K_SEG_LONG = 13     // and the long ones
+    K_SEG_LONG = 13,    // and the long ones
+    K_AXIS_COOP = 14    // k_axis whose blocks' warps share a split
 };
 enum Aux : uint8_t { AUX_NONE = 0, AUX_ARG = 1, AUX_PROD = 2 };
 
@@ -47,7 +48,7 @@ using CombineLaunch = cudaError_t (*)(const char* parts, int count, void* out, i
 struct KernelEntry {
     const void* fn;      // the __global__ function (occupancy queries)
     void* launch;        // one of the *Launch types above, by kind
-    int part_bytes = 0;  // K_AXIS, K_SEG_GROUP: bytes of one partial
+    int part_bytes = 0;  // K_AXIS, K_AXIS_COOP, K_SEG_GROUP: bytes of one partial
     int tile_slots = 0;  // K_REDUCE_TAIL: claimed tiles a block holds partials for
     int tile_loads = 0;  // K_REDUCE_TAIL: vectors a thread loads per round of a tile
 };
@@ -61,6 +62,9 @@ constexpr int kVecBytes[] = {16, 32};
 
 // Flat gradient of a row reduction (backward.cu); a.shift counts from the previous 32-byte boundary.
 cudaError_t launch_backward_flat(const BwdArgs& a, bool f64, cudaStream_t st);
+// Axis gradient by columns (backward.cu).
+cudaError_t launch_axis_backward_cols(const AxisBwdArgs& a, bool f64, int vb, int bx, int64_t groups, int64_t splits,
+                                      cudaStream_t st);
 
 void register_f32();
 void register_f32_seg();
