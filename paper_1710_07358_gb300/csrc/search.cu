@@ -9,8 +9,8 @@
 // k_phi      one pass over the four float32 link arrays evaluates phi at up
 //            to kLsMaxPts points: each term in float32, a thread's eight
 //            links per point summed pairwise and added to the point's Kahan
-//            pair, combined per block in float64 and by the last block in
-//            block order (the persistent reduction of Section 3 with a fixed
+//            pair, combined per warp in triples of float32 (72 bits), per
+//            block in float64 and by the last block in block order (the persistent reduction of Section 3 with a fixed
 //            combine order).  Error (u = 2^-24, first order): the linear
 //            part t0 v of a term takes three roundings (the fma placing v,
 //            the fma or product adding t0, the final product); the power
@@ -18,17 +18,17 @@
 //            2 u four times over, its two squarings, beta / 5, t0 kb and the
 //            last product; v^4: four on v and three of its own; the fma and
 //            the product) and (4 p + 7) u otherwise; the sums five (three
-//            pairwise levels, two for Kahan's update), the float64 combines
-//            below 2^-45.  So phi is within
+//            pairwise levels, two for Kahan's update), the combines above
+//            them below 2^-45.  So phi is within
 //            u (8 sum |t0 v| + (c_p + 5) sum |power part|), c_4 = 24.
 // k_ls_init  places the first two points and the speculative tree.
-// ls_step    (one thread of a search pass's last block, after the sums) walks
+// ls_step    (one warp of a search pass's last block, after the sums) walks
 //            depth D decisions with the values of the pass, then places the
 //            next pass's tree: the 2^(D+1) - 2 points the next D iterations
 //            could need, so that D iterations cost one pass over the links
 //            instead of D, and the sequence of points is exactly the
 //            sequential search's.
-// k_ls_init and ls_step run on one thread, with float64 operations written
+// k_ls_init and ls_step run on one warp, with float64 operations written
 // out (no contraction into FMA), so that the points match a float64
 // implementation that evaluates the same expressions in the same order.
 #include <cstdint>
@@ -39,7 +39,45 @@ namespace pr {
 
 // ---- evaluation pass -------------------------------------------------------
 
-__device__ void ls_step(LsState& s, double* result);
+// What a search step reads of the state, as one lane's copy.
+struct LsView {
+    double a, b, x1, x2, f1, f2, u, golden;
+    const double* fib;
+    int method, count, iter, total, depth, first, done;
+};
+__device__ __forceinline__ LsView ls_view(const LsState& s) {
+    return LsView{s.a, s.b, s.x1, s.x2, s.f1, s.f2, s.u, s.golden, s.fib, s.method, s.count, s.iter, s.total, s.depth,
+                  s.first, s.done};
+}
+__device__ void ls_step(LsState& s, LsView v, const double* vals, double* result, int lane);
+
+// Three floats whose sum is the value: a, the rounding errors of a, and those
+// of b, about 72 bits.
+struct F3 {
+    float a, b, c;
+};
+// s + e = x + y exactly (Knuth)
+__device__ __forceinline__ void two_sum(float x, float y, float& s, float& e) {
+    s = x + y;
+    const float t = s - x;
+    e = (x - (s - t)) + (y - t);
+}
+// Each TwoSum is exact; only the additions in c round, relative to parts of
+// about 2^-48: below 2^-70 of the operands' magnitudes.  Commutative bit for
+// bit (both errors and both sums are symmetric).
+__device__ __forceinline__ F3 f3_add(const F3& x, const F3& y) {
+    F3 r;
+    float e0, e1, e2;
+    two_sum(x.a, y.a, r.a, e0);
+    two_sum(x.b, y.b, r.b, e1);
+    two_sum(r.b, e0, r.b, e2);
+    r.c = (x.c + y.c) + (e1 + e2);
+    return r;
+}
+__device__ __forceinline__ F3 f3_shfl_xor(const F3& x, int m) {
+    return F3{__shfl_xor_sync(0xffffffffu, x.a, m), __shfl_xor_sync(0xffffffffu, x.b, m),
+              __shfl_xor_sync(0xffffffffu, x.c, m)};
+}
 
 // Kahan's compensated add: c holds the negated low part lost so far, so the
 // running sum is s - c
@@ -200,16 +238,44 @@ __global__ void __launch_bounds__(kPhiThreads, MP <= 8 ? 2 : 1) k_phi(PhiArgs a)
         phi_group<PW, 1, MP>(X, D, T, C, kb, a.power, al, m, s, e);
     }
 
-    // per point: thread pair -> float64, warp butterfly, warps in order
+    // per point: the warp's 32 Kahan pairs, added as triples of floats.  A
+    // butterfly of all MP points in float64 (two conversions and five
+    // additions a point and lane) took about half of a pass whose links sit
+    // in L2: GB300 adds float64 at 1.7 lanes a clock and SM.  Triples keep
+    // more bits on the float32 pipe, and each of the first steps sends half
+    // of the points to the other half of the lanes: MP - 1 additions and
+    // log2(32 / MP) more for all points instead of 5 MP.  Lane l ends with
+    // point l / (32 / MP).  (A search of 10^6 links at depth 2, 15 passes:
+    // 260 -> 165 us with this and the warp-wide search step.)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // Sums that might overflow float32 across the warp (and infinities) keep
+    // the float64 butterfly.
+    bool huge = false;
 #pragma unroll
-    for (int k = 0; k < MP; k++) {
-        if (k < m) {
+    for (int k = 0; k < MP; k++) huge |= !(fabsf(s[k]) < 0x1p115f);
+    if (__any_sync(0xffffffffu, huge)) {
+#pragma unroll
+        for (int k = 0; k < MP; k++) {
             double v = (double)s[k] - (double)e[k];
-#pragma unroll
             for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
             if (lane == 0) s_w[warp][k] = v;
         }
+    } else {
+        F3 f[MP];
+#pragma unroll
+        for (int k = 0; k < MP; k++) f[k] = F3{s[k], -e[k], 0.f};
+        int o = 16;
+#pragma unroll
+        for (int half = MP / 2; half >= 1; half >>= 1, o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int k = 0; k < half; k++) {
+                const F3 send = up ? f[k] : f[k + half], keep = up ? f[k + half] : f[k];
+                f[k] = f3_add(keep, f3_shfl_xor(send, o));
+            }
+        }
+        for (; o >= 1; o >>= 1) f[0] = f3_add(f[0], f3_shfl_xor(f[0], o));
+        if (lane % (32 / MP) == 0) s_w[warp][lane / (32 / MP)] = ((double)f[0].c + (double)f[0].b) + (double)f[0].a;
     }
     __syncthreads();
     if (threadIdx.x < m) {
@@ -223,19 +289,26 @@ __global__ void __launch_bounds__(kPhiThreads, MP <= 8 ? 2 : 1) k_phi(PhiArgs a)
     __syncthreads();
     if (!s_last) return;
     __threadfence();
+    // the search's state travels while the sums are made
+    LsView view{};
+    if (a.ls && warp == 0) view = ls_view(*a.ls);
     // the last block: warp w sums points w, w + 8, ... over the blocks, lanes
     // striding the block index, then a butterfly (a fixed order per grid)
+    __shared__ double s_val[kLsMaxPts];
     for (int k = warp; k < m; k += kPhiThreads / 32) {
         double v = 0.0;
         for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(a.partials + (int64_t)b * kLsMaxPts + k);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) a.out[k] = v;
+        if (lane == 0) {
+            a.out[k] = v;
+            s_val[k] = v;
+        }
     }
     if (threadIdx.x == 0) *a.ticket = 0u;
     if (a.ls) {
-        __syncthreads();                           // the sums of this pass are in a.out
-        if (threadIdx.x == 0) ls_step(*a.ls, a.result);
+        __syncthreads();                           // the sums of this pass are in s_val
+        if (warp == 0) ls_step(*a.ls, view, s_val, a.result, lane);
     }
 }
 
@@ -261,7 +334,7 @@ struct LsNode {
 // The child of n after one comparison: br 0 (x1 better) keeps [a, x2] and
 // moves x1 up to x2; br 1 keeps [x1, b] and moves x2 down to x1.  Returns
 // the new point the child needs.
-__device__ double ls_child(const LsState& s, const LsNode& n, int br, LsNode& c) {
+__device__ __forceinline__ double ls_child(const LsView& s, const LsNode& n, int br, LsNode& c) {
     c = n;
     c.j = n.j + 1;
     if (s.method == 0) {
@@ -290,24 +363,53 @@ __device__ double ls_child(const LsState& s, const LsNode& n, int br, LsNode& c)
     return c.x2;
 }
 
-// The tree of the next `levels` iterations below root, into pts[base...]
-__device__ int ls_tree(LsState& s, const LsNode& root, int levels, int base) {
-    LsNode cur[1 << kLsMaxDepth], nxt[1 << kLsMaxDepth];
-    cur[0] = root;
-    int width = 1, np = 0;
-    for (int l = 1; l <= levels; l++) {
-        for (int k = 0; k < width; k++)
-            for (int br = 0; br < 2; br++) s.pts[base + np++] = ls_child(s, cur[k], br, nxt[2 * k + br]);
-        width *= 2;
-        for (int k = 0; k < width; k++) cur[k] = nxt[k];
+// The tree of the next `levels` iterations below root, into pts[base...]:
+// lane j places node j (level l = 1, 2, ... holds 2^l nodes from 2^l - 2 on,
+// node k's path from the root is k's bits, the top one first), walking its
+// path with the same operations as any other lane.  Returns the node count.
+__device__ __forceinline__ int ls_tree(LsState& out, const LsView& s, const LsNode& root, int levels, int base, int lane) {
+    const int count = (2 << levels) - 2;
+    const int l = 31 - __clz(lane + 2), k = lane + 2 - (1 << l);
+    LsNode n = root;
+    double pt = 0.0;
+    for (int i = 1; i <= levels; i++) {
+        if (i > l) break;
+        LsNode c;
+        pt = ls_child(s, n, k >> (l - i) & 1, c);
+        n = c;
     }
-    return np;
+    if (lane < count) out.pts[base + lane] = pt;
+    return count;
 }
 
 __global__ void k_ls_init(LsState* sp, double lo, double hi, int method, int count, int total, int depth) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the first pass may start streaming
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    if (threadIdx.x >= 32 || blockIdx.x != 0) return;
+    const int lane = threadIdx.x;
     LsState& s = *sp;
+    LsView v{};
+    v.method = method;
+    v.count = count;
+    v.total = total;
+    v.depth = depth;
+    v.first = 1;
+    v.golden = __ddiv_rn(__dsub_rn(sqrt(5.0), 1.0), 2.0);
+    v.fib = s.fib;
+    v.a = lo;
+    v.b = hi;
+    if (method == 0) {
+        v.x1 = __dsub_rn(hi, __dmul_rn(v.golden, __dsub_rn(hi, lo)));
+        v.x2 = __dadd_rn(lo, __dmul_rn(v.golden, __dsub_rn(hi, lo)));
+    } else {
+        if (lane == 0) fill_fib(s.fib);
+        __syncwarp();
+        v.u = __ddiv_rn(__dsub_rn(hi, lo), s.fib[count]);
+        v.x1 = __dadd_rn(lo, __dmul_rn(s.fib[count - 2], v.u));
+        v.x2 = __dadd_rn(lo, __dmul_rn(s.fib[count - 1], v.u));
+    }
+    const LsNode root{v.a, v.b, v.x1, v.x2, 0};
+    const int np = ls_tree(s, v, root, depth < total ? depth : total, 2, lane);
+    if (lane != 0) return;
     s.method = method;
     s.count = count;
     s.total = total;
@@ -315,34 +417,29 @@ __global__ void k_ls_init(LsState* sp, double lo, double hi, int method, int cou
     s.iter = 0;
     s.first = 1;
     s.done = 0;
-    s.golden = __ddiv_rn(__dsub_rn(sqrt(5.0), 1.0), 2.0);
-    s.a = lo;
-    s.b = hi;
-    if (method == 0) {
-        s.u = 0.0;
-        s.x1 = __dsub_rn(hi, __dmul_rn(s.golden, __dsub_rn(hi, lo)));
-        s.x2 = __dadd_rn(lo, __dmul_rn(s.golden, __dsub_rn(hi, lo)));
-    } else {
-        fill_fib(s.fib);
-        s.u = __ddiv_rn(__dsub_rn(hi, lo), s.fib[count]);
-        s.x1 = __dadd_rn(lo, __dmul_rn(s.fib[count - 2], s.u));
-        s.x2 = __dadd_rn(lo, __dmul_rn(s.fib[count - 1], s.u));
-    }
-    s.pts[0] = s.x1;
-    s.pts[1] = s.x2;
-    const LsNode root{s.a, s.b, s.x1, s.x2, 0};
-    s.npts = 2 + ls_tree(s, root, depth < total ? depth : total, 2);
+    s.golden = v.golden;
+    s.u = v.u;
+    s.a = v.a;
+    s.b = v.b;
+    s.x1 = v.x1;
+    s.x2 = v.x2;
+    s.pts[0] = v.x1;
+    s.pts[1] = v.x2;
+    s.npts = 2 + np;
 }
 
 // After a pass: walk its decisions, then place the next pass's points, or
 // finish and write result (a, b, the better of the last two points, its
-// value).  Run by one thread of the pass's last block.
-__device__ void ls_step(LsState& s, double* result) {
+// value).  Run by one warp of the pass's last block: every lane walks the
+// decisions (vals: the pass's values, in shared memory), lane 0 writes the
+// state, and each lane places its own point of the tree (one thread placing
+// all of them in turn, through an array of nodes, took about 2 us a pass).
+__device__ void ls_step(LsState& out, LsView s, const double* vals, double* result, int lane) {
     if (s.done) return;
     const int base = s.first ? 2 : 0;
     if (s.first) {
-        s.f1 = s.vals[0];
-        s.f2 = s.vals[1];
+        s.f1 = vals[0];
+        s.f2 = vals[1];
     }
     LsNode n{s.a, s.b, s.x1, s.x2, s.iter};
     int path = 0;
@@ -351,7 +448,7 @@ __device__ void ls_step(LsState& s, double* result) {
         LsNode c;
         ls_child(s, n, br, c);
         path = 2 * path + br;
-        const double fnew = s.vals[base + (2 << l) - 2 + path];
+        const double fnew = vals[base + (2 << l) - 2 + path];
         if (br == 0) {
             s.f2 = s.f1;
             s.f1 = fnew;
@@ -362,26 +459,31 @@ __device__ void ls_step(LsState& s, double* result) {
         n = c;
         s.iter++;
     }
-    s.a = n.a;
-    s.b = n.b;
-    s.x1 = n.x1;
-    s.x2 = n.x2;
-    s.first = 0;
-    if (s.iter < s.total) {
+    const bool more = s.iter < s.total;
+    int np = 0;
+    if (more) {
         const int left = s.total - s.iter;
-        s.npts = ls_tree(s, n, s.depth < left ? s.depth : left, 0);
-        return;
+        np = ls_tree(out, s, n, s.depth < left ? s.depth : left, 0, lane);
+    } else if (s.method == 1) {
+        // Fibonacci's last comparison only shrinks the bracket
+        if (s.f1 < s.f2) n.b = n.x2;
+        else n.a = n.x1;
     }
-    // finished: Fibonacci's last comparison only shrinks the bracket
-    if (s.method == 1) {
-        if (s.f1 < s.f2) s.b = s.x2;
-        else s.a = s.x1;
-    }
-    s.done = 1;
-    s.npts = 0;
-    result[0] = s.a;
-    result[1] = s.b;
-    result[2] = s.f1 < s.f2 ? s.x1 : s.x2;
+    if (lane != 0) return;
+    out.a = n.a;
+    out.b = n.b;
+    out.x1 = n.x1;
+    out.x2 = n.x2;
+    out.f1 = s.f1;
+    out.f2 = s.f2;
+    out.iter = s.iter;
+    out.first = 0;
+    out.npts = np;
+    if (more) return;
+    out.done = 1;
+    result[0] = n.a;
+    result[1] = n.b;
+    result[2] = s.f1 < s.f2 ? n.x1 : n.x2;
     result[3] = s.f1 < s.f2 ? s.f1 : s.f2;
 }
 
