@@ -37,24 +37,24 @@ class RowReduce(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_out):
         op = ctx.op
-        rows, cols = ctx.shape
-        g = grad_out.contiguous()
         if op in ("max", "min"):
             (ai,) = ctx.saved_tensors
-            gi = pr.reduce_backward(op, _Shape(rows, cols), g, argidx=ai)
+            gi = pr.reduce_backward(op, _Shape(ctx.shape), grad_out, argidx=ai)
         elif op == "prod":
             x2d, ax = ctx.saved_tensors
-            gi = pr.reduce_backward(op, x2d, g, aux=ax)
+            gi = pr.reduce_backward(op, x2d, grad_out, aux=ax)
         else:
-            gi = pr.reduce_backward(op, _Shape(rows, cols), g)
+            gi = pr.reduce_backward(op, _Shape(ctx.shape), grad_out)
         return gi, None
 
 
 class _Shape:
     """Stands in for x where the backward needs only its shape."""
 
-    def __init__(self, *shape):
-        self.shape = tuple(shape)
+    __slots__ = ("shape",)
+
+    def __init__(self, shape):
+        self.shape = shape
 
     def data_ptr(self):
         return 0
@@ -76,23 +76,18 @@ class AxisReduce(torch.autograd.Function):
         else:
             raise ValueError("differentiable ops are sum, max, min and prod")
         ctx.op = op
-        ctx.dim = dim
-        ctx.shape = tuple(x.shape)
+        ctx.shape = x.shape
+        ctx.geometry = pr.axis_shape(x.shape, dim)
         return out
 
     @staticmethod
     def backward(ctx, grad_out):
-        op = ctx.op
-        g = grad_out.contiguous()
-        if op in ("max", "min"):
+        x = ai = ax = None
+        if ctx.op in ("max", "min"):
             (ai,) = ctx.saved_tensors
-            gi = pr.reduce_axis_backward(op, _Shape(*ctx.shape), ctx.dim, g, argidx=ai)
-        elif op == "prod":
+        elif ctx.op == "prod":
             x, ax = ctx.saved_tensors
-            gi = pr.reduce_axis_backward(op, x, ctx.dim, g, aux=ax)
-        else:
-            gi = pr.reduce_axis_backward(op, _Shape(*ctx.shape), ctx.dim, g)
-        return gi, None, None
+        return pr._axis_backward(ctx.op, ctx.shape, ctx.geometry, x, grad_out, ai, ax), None, None
 
 
 def reduce(x: torch.Tensor, op: str, dim: int = -1) -> torch.Tensor:

@@ -11,6 +11,7 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/pr.h"
@@ -26,18 +27,20 @@ namespace pr {
 // Kernel registry
 // ------------------------------------------------------------------------
 
-bool KernelKey::operator<(const KernelKey& o) const {
-    return std::tie(kind, dtype, op, prec, aux, unroll, vb) <
-           std::tie(o.kind, o.dtype, o.op, o.prec, o.aux, o.unroll, o.vb);
+// Keys pack into one word: a call looks up one to three kernels among some
+// two thousand.
+static uint64_t packed(const KernelKey& k) {
+    uint64_t v = 0;
+    for (uint8_t f : {k.kind, k.dtype, k.op, k.prec, k.aux, k.unroll, k.vb}) v = v << 8 | f;
+    return v;
 }
-
-static std::map<KernelKey, KernelEntry>& table() {
-    static std::map<KernelKey, KernelEntry> t;
+static std::unordered_map<uint64_t, KernelEntry>& table() {
+    static std::unordered_map<uint64_t, KernelEntry> t;
     return t;
 }
-void reg_add(const KernelKey& k, const KernelEntry& e) { table()[k] = e; }
+void reg_add(const KernelKey& k, const KernelEntry& e) { table()[packed(k)] = e; }
 const KernelEntry* reg_find(const KernelKey& k) {
-    auto it = table().find(k);
+    auto it = table().find(packed(k));
     return it == table().end() ? nullptr : &it->second;
 }
 

@@ -31,7 +31,6 @@ enum Aux : uint8_t { AUX_NONE = 0, AUX_ARG = 1, AUX_PROD = 2 };
 
 struct KernelKey {
     uint8_t kind, dtype, op, prec, aux, unroll, vb;
-    bool operator<(const KernelKey& o) const;
 };
 
 using ReduceLaunch = cudaError_t (*)(const ReduceArgs&, int grid, int block, cudaStream_t);

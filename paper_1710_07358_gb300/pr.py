@@ -14,6 +14,7 @@ first call raises.  There is no fallback.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -272,26 +273,46 @@ def check(status):
 # Tensor helpers
 # ---------------------------------------------------------------------------
 
+_T = None        # torch, on first use (the module loads without it)
+_RAW_STREAM = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _T, _RAW_STREAM
+    if _T is None:
+        import torch
+        _RAW_STREAM = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _T = torch
+    return _T
+
+
+_NAMES = {}      # torch dtype -> name
+_TDTYPES = {}    # name -> torch dtype (None where torch has none)
+
+
+def _tables():
+    torch = _torch()
+    for name, attr in (("f32", "float32"), ("f16", "float16"), ("bf16", "bfloat16"), ("f64", "float64"),
+                       ("i32", "int32"), ("i64", "int64"), ("u32", "uint32")):
+        t = getattr(torch, attr, None)
+        _TDTYPES[name] = t
+        if t is not None:
+            _NAMES[t] = name
 
 
 def dtype_name(t) -> str:
-    torch = _torch()
-    m = {torch.float32: "f32", torch.float16: "f16", torch.bfloat16: "bf16", torch.float64: "f64",
-         torch.int32: "i32", torch.int64: "i64"}
-    if hasattr(torch, "uint32"):
-        m[torch.uint32] = "u32"
-    if t.dtype not in m:
+    if not _NAMES:
+        _tables()
+    name = _NAMES.get(t.dtype)
+    if name is None:
         raise TypeError("unsupported tensor dtype %s" % t.dtype)
-    return m[t.dtype]
+    return name
 
 
 def torch_dtype(name: str):
-    torch = _torch()
-    return {"f32": torch.float32, "f16": torch.float16, "bf16": torch.bfloat16, "f64": torch.float64,
-            "i32": torch.int32, "i64": torch.int64, "u32": getattr(torch, "uint32", None)}[name]
+    if not _TDTYPES:
+        _tables()
+    return _TDTYPES[name]
 
 
 def out_dtype_name(dtype: str, op: str) -> str:
@@ -302,11 +323,25 @@ def out_dtype_name(dtype: str, op: str) -> str:
     return dtype
 
 
+_FORMS = {}      # (torch dtype, op) -> (dtype code, op code, output's torch dtype, output's dtype code)
+
+
+def _form(t, op):
+    """What a call on t under op needs of the tables, found once per (dtype, op)."""
+    d = dtype_name(t)
+    od = out_dtype_name(d, op)
+    f = _FORMS[t.dtype, op] = (DTYPES[d], OPS[op], torch_dtype(od), DTYPES[od])
+    return f
+
+
 def _stream(t, stream=None):
-    torch = _torch()
     if stream is not None:
         return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
-    return torch.cuda.current_stream(t.device).cuda_stream
+    # torch's own shortcut to the current stream's handle, where it has one:
+    # current_stream() makes a Stream object, 2 us a call against 0.1
+    if _RAW_STREAM is not None and t.is_cuda:
+        return _RAW_STREAM(t.get_device())
+    return _torch().cuda.current_stream(t.device).cuda_stream
 
 
 def _ptr(t):
@@ -315,17 +350,17 @@ def _ptr(t):
 
 def reduce(x, op: str, precision: str = "plain", out_dtype: str | None = None, out=None, stream=None):
     """0-d tensor holding the reduction of every element of the CUDA tensor x."""
-    torch = _torch()
     if not x.is_cuda:
         raise ValueError("reduce() needs a CUDA tensor; use reduce_host() for host memory")
     if not x.is_contiguous():
         raise ValueError("x must be contiguous")
-    d = dtype_name(x)
-    od = out_dtype or out_dtype_name(d, op)
+    dc, oc, tdt, odc = _FORMS.get((x.dtype, op)) or _form(x, op)
+    if out_dtype:
+        tdt, odc = torch_dtype(out_dtype), DTYPES[out_dtype]
     if out is None:
-        out = torch.empty((), dtype=torch_dtype(od), device=x.device)
-    check(pr_reduce_ex(_ptr(x), x.numel(), DTYPES[d], OPS[op], PRECISIONS[precision], DTYPES[od],
-                       _ptr(out), _stream(x, stream)))
+        out = _torch().empty((), dtype=tdt, device=x.device)
+    check((_lib or lib()).pr_reduce_ex(x.data_ptr(), x.numel(), dc, oc, PRECISIONS[precision], odc, out.data_ptr(),
+                                       _stream(x, stream)))
     return out
 
 
@@ -335,12 +370,13 @@ def reduce_arg(x, op: str, out=None, idx=None, stream=None):
     torch = _torch()
     if not x.is_cuda or not x.is_contiguous():
         raise ValueError("reduce_arg() needs a contiguous CUDA tensor")
-    d = dtype_name(x)
+    dc, oc, tdt, _ = _FORMS.get((x.dtype, op)) or _form(x, op)
     if out is None:
-        out = torch.empty((), dtype=torch_dtype(out_dtype_name(d, op)), device=x.device)
+        out = torch.empty((), dtype=tdt, device=x.device)
     if idx is None:
         idx = torch.empty((), dtype=torch.int64, device=x.device)
-    check(pr_reduce_arg(_ptr(x), x.numel(), DTYPES[d], OPS[op], _ptr(out), _ptr(idx), _stream(x, stream)))
+    check((_lib or lib()).pr_reduce_arg(x.data_ptr(), x.numel(), dc, oc, out.data_ptr(), idx.data_ptr(),
+                                        _stream(x, stream)))
     return out, idx
 
 
@@ -365,14 +401,13 @@ def segmented_reduce(x, offsets, op: str, precision: str = "plain", argidx: bool
     int8 tensor of nseg * 24 bytes (pr_prod_aux records), see prod_aux_fields().
     out / argidx_out / aux_out: caller-owned output tensors to write instead."""
     torch = _torch()
-    d = dtype_name(x)
+    dc, oc, tdt, _ = _FORMS.get((x.dtype, op)) or _form(x, op)
     nseg = offsets.numel() - 1
     if offsets.dtype != torch.int64 or not offsets.is_cuda or not offsets.is_contiguous():
         raise ValueError("offsets must be a contiguous int64 CUDA tensor")
-    out, ai, ax = _outputs(max(nseg, 0), torch_dtype(out_dtype_name(d, op)), x.device, argidx, aux, out,
-                           argidx_out, aux_out)
-    check(pr_segmented_reduce_aux(_ptr(x), _ptr(offsets), nseg, DTYPES[d], OPS[op], PRECISIONS[precision],
-                                  _ptr(out), _ptr(ai), _ptr(ax), _stream(x, stream)))
+    out, ai, ax = _outputs(max(nseg, 0), tdt, x.device, argidx, aux, out, argidx_out, aux_out)
+    check((_lib or lib()).pr_segmented_reduce_aux(x.data_ptr(), offsets.data_ptr(), nseg, dc, oc, PRECISIONS[precision],
+                                                  out.data_ptr(), _ptr(ai), _ptr(ax), _stream(x, stream)))
     if argidx:
         return out, ai
     if aux:
@@ -386,12 +421,11 @@ def reduce_rows(x, op: str, precision: str = "plain", argidx: bool = False, aux:
     (outputs as in segmented_reduce)."""
     if x.dim() != 2 or not x.is_contiguous():
         raise ValueError("reduce_rows needs a contiguous 2-D tensor")
-    d = dtype_name(x)
+    dc, oc, tdt, _ = _FORMS.get((x.dtype, op)) or _form(x, op)
     rows, cols = x.shape
-    out, ai, ax = _outputs(rows, torch_dtype(out_dtype_name(d, op)), x.device, argidx, aux, out, argidx_out,
-                           aux_out)
-    check(pr_reduce_rows(_ptr(x), rows, cols, DTYPES[d], OPS[op], PRECISIONS[precision], _ptr(out), _ptr(ai),
-                         _ptr(ax), _stream(x, stream)))
+    out, ai, ax = _outputs(rows, tdt, x.device, argidx, aux, out, argidx_out, aux_out)
+    check((_lib or lib()).pr_reduce_rows(x.data_ptr(), rows, cols, dc, oc, PRECISIONS[precision], out.data_ptr(),
+                                         _ptr(ai), _ptr(ax), _stream(x, stream)))
     if argidx:
         return out, ai
     if aux:
@@ -402,12 +436,12 @@ def reduce_rows(x, op: str, precision: str = "plain", argidx: bool = False, aux:
 def scan(x, op: str, exclusive: bool = False, out=None, stream=None):
     """Prefix scan of a contiguous CUDA tensor (flattened) under op; same
     number of elements, in the output type of the reduction (pr_out_dtype)."""
-    torch = _torch()
     if not x.is_cuda or not x.is_contiguous():
         raise ValueError("scan needs a contiguous CUDA tensor")
-    d = dtype_name(x)
-    y = out if out is not None else torch.empty(x.shape, dtype=torch_dtype(out_dtype_name(d, op)), device=x.device)
-    check(pr_scan(_ptr(x), x.numel(), DTYPES[d], OPS[op], 1 if exclusive else 0, _ptr(y), _stream(x, stream)))
+    dc, oc, tdt, _ = _FORMS.get((x.dtype, op)) or _form(x, op)
+    y = out if out is not None else _torch().empty(x.shape, dtype=tdt, device=x.device)
+    check((_lib or lib()).pr_scan(x.data_ptr(), x.numel(), dc, oc, 1 if exclusive else 0, y.data_ptr(),
+                                  _stream(x, stream)))
     return y
 
 
@@ -464,13 +498,7 @@ def line_search(x, d, t0, cap, lo: float = 0.0, hi: float = 1.0, beta: float = 0
 def axis_shape(shape, dim):
     """(outer, n, inner) of a reduction of `dim` over a contiguous tensor of `shape`."""
     dim = dim % len(shape)
-    outer = 1
-    for v in shape[:dim]:
-        outer *= v
-    inner = 1
-    for v in shape[dim + 1:]:
-        inner *= v
-    return outer, shape[dim], inner
+    return math.prod(shape[:dim]), shape[dim], math.prod(shape[dim + 1:])
 
 
 def reduce_axis(x, op: str, dim: int, precision: str = "plain", argidx: bool = False, aux: bool = False,
@@ -483,17 +511,19 @@ def reduce_axis(x, op: str, dim: int, precision: str = "plain", argidx: bool = F
     torch = _torch()
     if not x.is_cuda or not x.is_contiguous():
         raise ValueError("reduce_axis needs a contiguous CUDA tensor")
-    d = dtype_name(x)
-    outer, n, inner = axis_shape(tuple(x.shape), dim)
-    oshape = tuple(v for i, v in enumerate(x.shape) if i != dim % x.dim())
+    dc, oc, tdt, _ = _FORMS.get((x.dtype, op)) or _form(x, op)
+    shape = tuple(x.shape)
+    outer, n, inner = axis_shape(shape, dim)
+    dim %= len(shape)
+    oshape = shape[:dim] + shape[dim + 1:]
     if out is None:
-        out = torch.empty(oshape, dtype=torch_dtype(out_dtype_name(d, op)), device=x.device)
+        out = torch.empty(oshape, dtype=tdt, device=x.device)
     ai = (argidx_out if argidx_out is not None else torch.empty(oshape, dtype=torch.int64, device=x.device)) \
         if argidx else None
     ax = (aux_out if aux_out is not None else torch.empty(outer * inner * 24, dtype=torch.int8, device=x.device)) \
         if aux else None
-    check(pr_reduce_axis(_ptr(x), outer, n, inner, DTYPES[d], OPS[op], PRECISIONS[precision], _ptr(out), _ptr(ai),
-                         _ptr(ax), _stream(x, stream)))
+    check((_lib or lib()).pr_reduce_axis(x.data_ptr(), outer, n, inner, dc, oc, PRECISIONS[precision], out.data_ptr(),
+                                         _ptr(ai), _ptr(ax), _stream(x, stream)))
     if argidx:
         return out, ai
     if aux:
@@ -504,14 +534,18 @@ def reduce_axis(x, op: str, dim: int, precision: str = "plain", argidx: bool = F
 def reduce_axis_backward(op: str, x, dim: int, grad_out, argidx=None, aux=None, out=None, stream=None):
     """grad_in (x's shape) for reduce_axis(x, op, dim); x is read only for prod
     (anything with .shape and .data_ptr() serves otherwise)."""
-    torch = _torch()
-    d = dtype_name(grad_out)
     shape = tuple(x.shape)
-    outer, n, inner = axis_shape(shape, dim)
-    gi = out if out is not None else torch.empty(shape, dtype=grad_out.dtype, device=grad_out.device)
-    xp = _ptr(x) if op == "prod" else None
-    check(pr_reduce_axis_backward(OPS[op], DTYPES[d], xp, outer, n, inner, _ptr(grad_out.contiguous()),
-                                  _ptr(argidx), _ptr(aux), _ptr(gi), _stream(grad_out, stream)))
+    return _axis_backward(op, shape, axis_shape(shape, dim), x if op == "prod" else None, grad_out, argidx, aux, out, stream)
+
+
+def _axis_backward(op, shape, geometry, x, grad_out, argidx=None, aux=None, out=None, stream=None):
+    """reduce_axis_backward with its geometry (outer, n, inner) at hand."""
+    dc, oc, _, _ = _FORMS.get((grad_out.dtype, op)) or _form(grad_out, op)
+    outer, n, inner = geometry
+    gi = out if out is not None else _torch().empty(shape, dtype=grad_out.dtype, device=grad_out.device)
+    g = grad_out.contiguous()
+    check((_lib or lib()).pr_reduce_axis_backward(oc, dc, _ptr(x), outer, n, inner, g.data_ptr(), _ptr(argidx), _ptr(aux),
+                                                  gi.data_ptr(), _stream(grad_out, stream)))
     return gi
 
 
@@ -524,13 +558,12 @@ def prod_aux_fields(aux):
 
 def reduce_backward(op: str, x, grad_out, argidx=None, aux=None, out=None, stream=None):
     """grad_in [rows, cols] for a row reduction of x (see pr_reduce_backward)."""
-    torch = _torch()
-    d = dtype_name(grad_out)
+    dc, oc, _, _ = _FORMS.get((grad_out.dtype, op)) or _form(grad_out, op)
     rows, cols = x.shape
-    gi = out if out is not None else torch.empty((rows, cols), dtype=grad_out.dtype, device=grad_out.device)
-    xp = _ptr(x) if op == "prod" else None
-    check(pr_reduce_backward(OPS[op], DTYPES[d], xp, rows, cols, _ptr(grad_out.contiguous()), _ptr(argidx),
-                             _ptr(aux), _ptr(gi), _stream(grad_out, stream)))
+    gi = out if out is not None else _torch().empty((rows, cols), dtype=grad_out.dtype, device=grad_out.device)
+    g = grad_out.contiguous()
+    check((_lib or lib()).pr_reduce_backward(oc, dc, x.data_ptr() if op == "prod" else None, rows, cols, g.data_ptr(),
+                                             _ptr(argidx), _ptr(aux), gi.data_ptr(), _stream(grad_out, stream)))
     return gi
 
 
