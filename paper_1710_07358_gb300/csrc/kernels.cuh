@@ -47,9 +47,9 @@
 //   first kernel takes up to 32 neighbouring segments a warp, through shared
 //   memory where they are short; the second shares the long ones among all
 //   warps, chunk by chunk.  fp32 sum on GB300: 10^6 segments of 24 elements on
-//   average (96 MB) 841 -> 52 us (0.30 of a 6.8 TB/s copy), 65536 of 1000 230
+//   average (96 MB) 841 -> 50 us (0.31 of a 6.8 TB/s copy), 65536 of 1000 230
 //   -> 64, 10^5 log-uniform to 16384 316 -> 202, 8192 of 40000 207 -> 207;
-//   maximum with index of the first 976 -> 107, of the last 538 -> 243.  Short
+//   maximum with index of the first 976 -> 105, of the last 538 -> 243.  Short
 //   segments are bound by instructions, about 24 warp instructions a segment
 //   of 24 (ncu: issue slots 60 % busy, no one stall dominant), long ones by HBM.
 //
@@ -1301,8 +1301,8 @@ __device__ __forceinline__ Segs seg_bounds(const int64_t* off, int64_t nseg) {
 // shared memory that the L1 cache needs for the loads in flight of the direct
 // path and of k_seg_long (measured: 8192 segments of 40000 254 us with two
 // stages, 207 with one).  Five blocks an SM: 96 registers, the most that no
-// trait on the fp32 path spills at (10^6 segments of 24: 52 us; six blocks 53,
-// eight 53, and 118 against 106 for the maximum with index).
+// trait on the fp32 path spills at (10^6 segments of 24: 50 us; six blocks 53,
+// eight 53; 105 against 107 and 118 for the maximum with index).
 constexpr int kSegBlock = 128;
 constexpr int kStageBytes = 4096;    // a warp's stage: one batch
 constexpr int kStageMean = 512;
@@ -1373,17 +1373,21 @@ __global__ void __launch_bounds__(kSegBlock, 5) k_seg_group(SegGroupArgs a) {
                     const int len = __shfl_sync(kAll, n0, i);
                     ShortAcc<T> acc;
                     int j = t;
-                    if constexpr (!T::kIdx && !kWidePart<T>) {
-                        // four at a time, summed pairwise: a shorter chain of
-                        // operations and of roundings
-                        for (; j + 3 * lanes < len; j += 4 * lanes) {
-                            const typename Ld::E e[4] = {Ld::lone(run[j]), Ld::lone(run[j + lanes]),
-                                                         Ld::lone(run[j + 2 * lanes]), Ld::lone(run[j + 3 * lanes])};
+                    for (; j + 3 * lanes < len; j += 4 * lanes) {
+                        const typename Ld::E e[4] = {Ld::lone(run[j]), Ld::lone(run[j + lanes]),
+                                                     Ld::lone(run[j + 2 * lanes]), Ld::lone(run[j + 3 * lanes])};
+                        // (summed pairwise: a shorter chain of operations and
+                        // of roundings)
+                        if constexpr (!T::kIdx && !kWidePart<T>) {
                             acc.add_vec(e, 0);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; q++) acc.add(e[q], j + q * lanes);
                         }
                     }
-#pragma unroll 4
-                    for (; j < len; j += lanes) acc.add(Ld::lone(run[j]), j);
+#pragma unroll
+                    for (int q = 0; q < 3; q++)
+                        if (j + q * lanes < len) acc.add(Ld::lone(run[j + q * lanes]), j + q * lanes);
                     const Part p = group_combine<T>(acc.part(), gl);
                     if (t == 0 && len > 0) store_segment<T>(p, s0 + i, a.out, a.argidx, a.aux);
                 }
