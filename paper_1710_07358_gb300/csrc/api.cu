@@ -715,17 +715,18 @@ static pr_status axis_scratch(cudaStream_t st, size_t bytes, char** out) {
 
 // Row splits of `tiles` blocks' worth of work with `resident` blocks at once:
 // the least estimated time.  The input streams in stream_us when the waves of
-// blocks are full (a single wave streams at full rate from about 0.6 of the
-// GPU on); SMs that finish early cost about 0.08 of a wave ([16, 4096, 4096]
-// fp32 sum: 173 us in one wave, 160 in many); a wave about 2 us to start and
-// to combine, a finishing pass as much; the partials `part` of the input's
-// traffic per split.
+// blocks are full (a single wave from 0.9 of the GPU on: with 0.6, which took
+// two splits for three, [64, 577, 768] fp32 maximum with index 33.4 us against
+// 30.7, [3, 10000, 256] fp64 product 36.5 against 22.9); SMs that finish early
+// cost about 0.08 of a wave ([16, 4096, 4096] fp32 sum: 173 us in one wave,
+// 160 in many); a wave about 2 us to start and to combine, a finishing pass as
+// much; the partials `part` of the input's traffic per split.
 static int64_t axis_splits(int64_t tiles, int64_t resident, int64_t most, double stream_us, double part) {
     int64_t best = 1;
     double least = 1e30;
     for (int64_t s = 1; s <= most && s <= 1024; s++) {
         const double w = (double)tiles * s / (double)resident, waves = std::ceil(w);
-        const double fill = w <= 1.0 ? (0.6 / w > 1.0 ? 0.6 / w : 1.0) : waves / w;
+        const double fill = w <= 1.0 ? (0.9 / w > 1.0 ? 0.9 / w : 1.0) : waves / w;
         const double us = stream_us * (fill + 0.08 / waves + (s > 1 ? part * s : 0.0)) + 2.0 * waves + (s > 1 ? 2.0 : 0.0);
         if (us < least) {
             least = us;
@@ -742,7 +743,7 @@ static int64_t axis_splits(int64_t tiles, int64_t resident, int64_t most, double
 // those come to more than a twentieth of the input's traffic, the warps of a
 // block share a split instead, and axis_splits has their number (measured on
 // GB300, us: [64, 577, 768] fp32 maximum with index 77 with 49 splits of a
-// warp, 33 shared; [4096, 16, 512] sum 44 and 29; [16, 4096, 4096] sum 159 and
+// warp, 31 shared; [4096, 16, 512] sum 44 and 32; [16, 4096, 4096] sum 159 and
 // 166, maximum 168 and 199).  Inputs below 7 MB are bound by latency either
 // way, and columns that are not whole vectors keep more rows in flight in the
 // smaller kernel ([1, 5000, 4099] maximum 49 and 57).  splits > 1 add a

@@ -16,8 +16,8 @@
 //   warp order), and only then are the rows split over blocks: a partial per
 //   warp and output cost more traffic than the input where the axis is short
 //   ([64, 577, 768] fp32 maximum with index: 49 splits wrote and read 38 MB
-//   each of 16-byte partials for 113 MB of input; with shared splits 77 -> 33
-//   us, 0.51 of a 6.8 TB/s copy: one wave of blocks, bound by latency).  With one split the outputs
+//   each of 16-byte partials for 113 MB of input; with shared splits 77 -> 31
+//   us, 0.54 of a 6.8 TB/s copy: one wave of blocks, bound by latency).  With one split the outputs
 //   are written; with more, the partials, and k_axis_finish combines each output's
 //   partials in a fixed order (one thread per output folding the splits in
 //   order, or with many splits one warp per output and a fixed tree), so
