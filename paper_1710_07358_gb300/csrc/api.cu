@@ -211,8 +211,9 @@ static pr_status get_ws(cudaStream_t st, Workspace* out) {
     ws.blk_done = u + gmax + 2;
     ws.err = reinterpret_cast<int*>(u + gmax + 32);
     ws.gmax = gmax;
-    ws.task_count = u + gmax + 3;
-    ws.tasks = reinterpret_cast<SegTask*>(u + gmax + 64);   // (16-byte aligned: gmax is a multiple of 32)
+    // (8- and 16-byte aligned: gmax is a multiple of 32)
+    ws.task_count = reinterpret_cast<SegCount*>(u + gmax + 4);
+    ws.tasks = reinterpret_cast<SegTask*>(u + gmax + 64);
     g_ws[key] = WsRec{ws, base, bytes};
     *out = ws;
     return PR_OK;
@@ -512,7 +513,7 @@ static pr_status run_seg_group(const void* x, const int64_t* off, int64_t nseg, 
     const bool injected = inject(PR_FAULT_LAUNCH);
     if (!injected) err = reinterpret_cast<SegGroupLaunch>(el->launch)(a, di.sms * occ_l, kGroupBlock, st);
     if (injected || err != cudaSuccess) {
-        cudaMemsetAsync(ws.task_count, 0, sizeof(unsigned), st);   // the list is for this call only
+        cudaMemsetAsync(ws.task_count, 0, sizeof(SegCount), st);   // the list is for this call only
         if (injected) return fail(PR_ERR_CUDA, "kernel launch failed (injected by the test hook)");
         return fail(PR_ERR_CUDA, "segmented launch: %s", cudaGetErrorString(err));
     }

@@ -78,6 +78,7 @@
 // k_combine_parts  one block combining an array of partials in order.
 #pragma once
 #include <type_traits>
+#include "segtasks.h"
 #include "traits.cuh"
 
 namespace pr {
@@ -126,7 +127,7 @@ struct Workspace {
     int* err;            // device error word
     int gmax;
     SegTask* tasks = nullptr;       // kSegTasks (k_seg_group)
-    unsigned* task_count = nullptr; // tasks listed, zero between launches
+    SegCount* task_count = nullptr; // tasks asked for, zero between launches
 };
 
 struct ReduceArgs {
@@ -1263,23 +1264,6 @@ __global__ void __launch_bounds__(512) k_segmented(SegArgs a) {
 // Many segments
 // ------------------------------------------------------------------------
 
-// A segment of more than `most` elements is left to k_seg_long, in chunks of
-// `chunk`.  Both grow with the elements so that the tasks fit: at most half
-// of them long segments (unless there are that few segments at all), the
-// other half the further chunks of those.
-constexpr int64_t kLongSeg = 2048;
-constexpr int64_t kLongChunk = 8192;
-
-struct SegSplit {
-    int64_t most, chunk;
-};
-__device__ __forceinline__ SegSplit seg_split_lengths(int64_t total, int64_t nseg, unsigned tasks) {
-    const int64_t share = total / (tasks / 2) + 1;
-    const int64_t most = nseg <= tasks / 2 || share < kLongSeg ? kLongSeg : share;
-    const int64_t chunk = share < kLongChunk ? kLongChunk : share;
-    return {most, chunk < most ? most : chunk};
-}
-
 __device__ __forceinline__ Segs seg_bounds(const int64_t* off, int64_t nseg) {
     Segs sg{off, 0, nseg, 0, 0};
     const int64_t raw0 = sg.raw(0), rawN = sg.raw(nseg);
@@ -1401,13 +1385,16 @@ __global__ void __launch_bounds__(kSegBlock, 5) k_seg_group(SegGroupArgs a) {
         if (mine && len == 0) T::store_empty(a.out, s0 + lane, false, a.argidx, a.aux);
         unsigned big = __ballot_sync(kAll, len > sp.most);
         if (big) {
-            const unsigned n = big >> lane & 1u ? (unsigned)((len + sp.chunk - 1) / sp.chunk) : 0u;
-            const unsigned first = n ? atomicAdd(a.ws.task_count, n) : 0u;
+            const unsigned n = big >> lane & 1u ? seg_chunks(len, sp) : 0u;
+            const SegCount first = n ? atomicAdd(a.ws.task_count, (SegCount)n) : 0u;
+            // (malformed offsets may ask for more tasks than there are: the
+            // segments past the end of the list stay unset)
+            const unsigned listed = seg_listed(first, n, a.tasks);
+            if (listed < n) atomicOr(a.ws.err, kErrInvalid);
             for (; big; big &= big - 1) {
                 const int i = __ffs(big) - 1;
-                const unsigned f = __shfl_sync(kAll, first, i), c = __shfl_sync(kAll, n, i);
-                // (malformed offsets may list more: those segments stay unset)
-                for (unsigned k = lane; k < c && f + k < a.tasks; k += 32) a.ws.tasks[f + k] = SegTask{s0 + i, f, 0u};
+                const unsigned f = __shfl_sync(kAll, (unsigned)first, i), c = __shfl_sync(kAll, listed, i);
+                for (unsigned k = lane; k < c; k += 32) a.ws.tasks[f + k] = SegTask{s0 + i, f, 0u};
             }
         }
         warp_segments<T>(x, a.shift, sg.P0, sg.P1, s0, b, len > 0 && len <= sp.most ? (int)len : 0, gl, a.out, a.argidx,
@@ -1431,8 +1418,8 @@ __global__ void __launch_bounds__(kGroupBlock) k_seg_long(SegGroupArgs a) {
     const SegSplit sp = seg_split_lengths(sg.P1 - sg.P0, a.nseg, a.tasks);
     const int lane = threadIdx.x & 31;
     asm volatile("griddepcontrol.wait;" ::: "memory");   // k_seg_group is done and its list visible
-    const unsigned listed = __ldcg(a.ws.task_count);
-    const unsigned ntask = listed < a.tasks ? listed : a.tasks;
+    const SegCount asked = __ldcg(a.ws.task_count);
+    const unsigned ntask = asked < a.tasks ? (unsigned)asked : a.tasks;
     Part* parts = reinterpret_cast<Part*>(a.ws.head);
     auto claim = [&]() { return lane == 0 ? atomicAdd(a.ws.chunk_ctr, 1u) : 0u; };
     auto record = [&](unsigned k, int64_t& s, unsigned& first) {
@@ -1453,7 +1440,7 @@ __global__ void __launch_bounds__(kGroupBlock) k_seg_long(SegGroupArgs a) {
             record(k1, s1, first1);
             const unsigned c = k - first;                    // this chunk of the segment
             const int64_t len = e - b, c0 = (int64_t)c * sp.chunk, left = len - c0;
-            const unsigned chunks = (unsigned)((len + sp.chunk - 1) / sp.chunk);
+            const unsigned chunks = seg_chunks(len, sp);
             Part p = group_part<T, 4>(x, b + c0, (int)(left < sp.chunk ? left : sp.chunk), a.shift, sg.P0, sg.P1, lane,
                                       32, c0);
             const int64_t b1 = sg.begin(s1), e1 = sg.end(s1);
@@ -1512,7 +1499,7 @@ __global__ void __launch_bounds__(kGroupBlock) k_seg_long(SegGroupArgs a) {
         __threadfence();
         if (atomicAdd(a.ws.blk_done, 1u) == gridDim.x - 1) {
             *a.ws.chunk_ctr = 0u;
-            *a.ws.task_count = 0u;
+            *a.ws.task_count = 0;
             *a.ws.blk_done = 0u;
         }
     }
