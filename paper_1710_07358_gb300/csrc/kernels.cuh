@@ -1051,7 +1051,7 @@ __global__ void __launch_bounds__(512) k_segmented(SegArgs a) {
             const int64_t nwarp = nth >> 5;
             int batch = 5;
             while (batch > 0 && (nseg >> batch) < nwarp) batch--;
-            segment_batches<T>(sg, x, (int)(reinterpret_cast<uintptr_t>(x) % kGroupVec) / Ld::ES, batch, gtid >> 5,
+            segment_batches<typename GroupTrait<T>::type>(sg, x, (int)(reinterpret_cast<uintptr_t>(x) % kGroupVec) / Ld::ES, batch, gtid >> 5,
                                nwarp, kGroupMost, a.out, a.argidx, a.aux, a.ws.err);
             return;
         }

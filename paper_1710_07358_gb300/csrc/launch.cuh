@@ -130,15 +130,16 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
     reg_one<T, 4, 16>(dtype, op, prec, aux, plain, seg);
     reg_one<T, 4, 32>(dtype, op, prec, aux, plain, seg);
     if (seg) {
+        using G = typename GroupTrait<T>::type;
         reg_add(KernelKey{K_ROWS_GROUP, dtype, op, prec, aux, 0, 0},
-                KernelEntry{reinterpret_cast<const void*>(&k_rows_group<T>),
-                            reinterpret_cast<void*>(&launch_rows_group<T>)});
-        KernelEntry sg{reinterpret_cast<const void*>(&k_seg_group<T>), reinterpret_cast<void*>(&launch_seg_group<T>)};
-        sg.part_bytes = (int)sizeof(typename T::Part);
+                KernelEntry{reinterpret_cast<const void*>(&k_rows_group<G>),
+                            reinterpret_cast<void*>(&launch_rows_group<G>)});
+        KernelEntry sg{reinterpret_cast<const void*>(&k_seg_group<G>), reinterpret_cast<void*>(&launch_seg_group<G>)};
+        sg.part_bytes = (int)sizeof(typename G::Part);
         reg_add(KernelKey{K_SEG_GROUP, dtype, op, prec, aux, 0, 0}, sg);
         reg_add(KernelKey{K_SEG_LONG, dtype, op, prec, aux, 0, 0},
-                KernelEntry{reinterpret_cast<const void*>(&k_seg_long<T>),
-                            reinterpret_cast<void*>(&launch_seg_long<T>)});
+                KernelEntry{reinterpret_cast<const void*>(&k_seg_long<G>),
+                            reinterpret_cast<void*>(&launch_seg_long<G>)});
         reg_axis<T, 2, 0>(dtype, op, prec, aux);
         reg_axis<T, 2, 16>(dtype, op, prec, aux);
         reg_axis<T, 2, 32>(dtype, op, prec, aux);

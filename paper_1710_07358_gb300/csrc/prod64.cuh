@@ -108,4 +108,14 @@ struct ProdMix {
     }
 };
 
+// Groups of lanes multiply on the integer pipes alone: half of a lane's factors
+// would round on the fp64 pipe, where the short runs that groups take used to
+// meet an element or a vector a thread and round once or not at all (relative
+// error, [32768, 1000] 1.1e-15 against 8.0e-16 by k_rows, [30000, 1001]
+// 1.1e-15 against 8.7e-17 by k_segmented; 8.7e-17 now).
+template <>
+struct GroupTrait<ProdMix> {
+    using type = ProdExt;
+};
+
 }  // namespace pr

@@ -134,6 +134,15 @@ struct LdI64 {
     __device__ __forceinline__ static E lone(In v) { return (uint64_t)v; }
 };
 
+// The trait with which groups of lanes reduce a run (k_rows_group, k_seg_group,
+// k_seg_long, k_segmented's short segments).  A lane of a group adds far more
+// elements than a thread of a wide block, so a trait whose error grows with a
+// thread's own elements names one with the same Part and a longer accumulator.
+template <class T>
+struct GroupTrait {
+    using type = T;
+};
+
 // Output writers for float-valued results.
 __device__ __forceinline__ void put_f32(void* out, int64_t i, float v) { static_cast<float*>(out)[i] = v; }
 __device__ __forceinline__ void put_f64(void* out, int64_t i, double v) { static_cast<double*>(out)[i] = v; }
