@@ -678,50 +678,6 @@ struct GroupAccs {
     static constexpr int value = sizeof(typename T::Acc) <= 8 ? U : 1;
 };
 
-// An fp32 accumulator whose Part is a double (FP64_COMBINE).  A lane of a
-// group adds more elements than a thread of a wide block does, and the mode
-// is there to keep fp32 chains short, so groups join it to the double part
-// often: after every few vectors of long runs, after every element of short
-// ones.
-template <class T>
-constexpr bool kWidePart = sizeof(typename T::Acc) == 4 && sizeof(typename T::Part) == 8;
-
-// Accumulation of a short run, an element or a few neighbours at a time.
-template <class T>
-struct ShortAcc {
-    using A = std::conditional_t<kWidePart<T>, typename T::Part, typename T::Acc>;
-    A a;
-    __device__ __forceinline__ ShortAcc() {
-        if constexpr (kWidePart<T>) a = T::part_init();
-        else a = T::init();
-    }
-    __device__ __forceinline__ void add(typename T::Ld::E e, int i) {
-        if constexpr (kWidePart<T>) {
-            typename T::Acc one = T::init();
-            T::add(one, e, i);
-            a = T::combine(a, T::to_part(one));
-        } else {
-            T::add(a, e, i);
-        }
-    }
-    // N elements with indices from i on, summed as a tree (a trait without
-    // indices takes any N elements)
-    template <int N>
-    __device__ __forceinline__ void add_vec(const typename T::Ld::E (&e)[N], int i) {
-        if constexpr (kWidePart<T>) {
-            typename T::Acc one = T::init();
-            T::add_vec(one, e, i);
-            a = T::combine(a, T::to_part(one));
-        } else {
-            T::add_vec(a, e, i);
-        }
-    }
-    __device__ __forceinline__ typename T::Part part() const {
-        if constexpr (kWidePart<T>) return a;
-        else return T::to_part(a);
-    }
-};
-
 // The elements [p0, p0 + len) of x that lane t of G neighbours takes, combined
 // into one Part (the trait is given indices relative to p0, plus i0).  The run is
 // covered by 32-byte vectors on the 32-byte grid of memory, lane t taking
@@ -736,7 +692,6 @@ __device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In*
     using E = typename Ld::E;
     constexpr int VE = kGroupVec / Ld::ES;
     constexpr int NA = GroupAccs<T, U>::value;
-    typename T::Part wide = T::part_init();
     typename T::Acc acc[NA];
 #pragma unroll
     for (int u = 0; u < NA; u++) acc[u] = T::init();
@@ -773,14 +728,8 @@ __device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In*
                 for (int i = c > 0 ? c : 0; i < e1; i++) T::add(a, Ld::one(x, p0 + i), i0 + i);
             }
         }
-        if constexpr (kWidePart<T>) {
-            wide = T::combine(wide, fold<T, NA>(acc));
-#pragma unroll
-            for (int u = 0; u < NA; u++) acc[u] = T::init();
-        }
     }
-    if constexpr (kWidePart<T>) return wide;
-    else return fold<T, NA>(acc);
+    return fold<T, NA>(acc);
 }
 
 // Combine across the lanes of each group of 2^gl neighbours (gl <= 5; all 32
@@ -843,7 +792,7 @@ __device__ __forceinline__ void warp_segments(const typename T::Ld::In* x, int s
         const int mis = (int)((p0 + shift) & (VE - 1));
         const int nv = n > 0 ? (n + mis + VE - 1) / VE : 0;
         const typename Ld::In* base = x + (p0 - mis);
-        ShortAcc<T> acc;
+        typename T::Acc acc = T::init();
         for (int j = t; __any_sync(kAll, j < nv); j += U * lanes) {
             Words<kGroupVec> w[U];
 #pragma unroll
@@ -859,15 +808,15 @@ __device__ __forceinline__ void warp_segments(const typename T::Ld::In* x, int s
                 const int lo = c < 0 ? -c : 0, hi = n - c;
                 const unsigned m = (hi >= VE ? (unsigned)((1ull << VE) - 1) : (1u << hi) - 1u) >> lo << lo;
                 if (c >= 0 && hi >= VE) {
-                    acc.add_vec(e, c);
+                    T::add_vec(acc, e, c);
                 } else {
 #pragma unroll
                     for (int q = 0; q < VE; q++)
-                        if (m >> q & 1u) acc.add(e[q], c + q);
+                        if (m >> q & 1u) T::add(acc, e[q], c + q);
                 }
             }
         }
-        const Part p = group_combine<T>(acc.part(), gl);
+        const Part p = group_combine<T>(T::to_part(acc), gl);
         if (t == 0 && n > 0) store_segment<T>(p, s0 + i, out, argidx, aux);
         if (k + per >= 32) break;
     }
@@ -1355,24 +1304,24 @@ __global__ void __launch_bounds__(kSegBlock, 5) k_seg_group(SegGroupArgs a) {
                     const int i = k + (lane >> gl);
                     const In* run = v + __shfl_sync(kAll, r0, i);
                     const int len = __shfl_sync(kAll, n0, i);
-                    ShortAcc<T> acc;
+                    typename T::Acc acc = T::init();
                     int j = t;
                     for (; j + 3 * lanes < len; j += 4 * lanes) {
                         const typename Ld::E e[4] = {Ld::lone(run[j]), Ld::lone(run[j + lanes]),
                                                      Ld::lone(run[j + 2 * lanes]), Ld::lone(run[j + 3 * lanes])};
                         // (summed pairwise: a shorter chain of operations and
                         // of roundings)
-                        if constexpr (!T::kIdx && !kWidePart<T>) {
-                            acc.add_vec(e, 0);
+                        if constexpr (!T::kIdx) {
+                            T::add_vec(acc, e, 0);
                         } else {
 #pragma unroll
-                            for (int q = 0; q < 4; q++) acc.add(e[q], j + q * lanes);
+                            for (int q = 0; q < 4; q++) T::add(acc, e[q], j + q * lanes);
                         }
                     }
 #pragma unroll
                     for (int q = 0; q < 3; q++)
-                        if (j + q * lanes < len) acc.add(Ld::lone(run[j + q * lanes]), j + q * lanes);
-                    const Part p = group_combine<T>(acc.part(), gl);
+                        if (j + q * lanes < len) T::add(acc, Ld::lone(run[j + q * lanes]), j + q * lanes);
+                    const Part p = group_combine<T>(T::to_part(acc), gl);
                     if (t == 0 && len > 0) store_segment<T>(p, s0 + i, a.out, a.argidx, a.aux);
                 }
                 __syncwarp();

@@ -186,6 +186,46 @@ struct SumF {
     }
 };
 
+// The sum's group form: a lane keeps two running sums (two chains of dependent
+// additions) and, apart from them, the sums of the exact rounding errors of
+// their additions (Knuth's TwoSum); they meet in fp32 the same way, and once,
+// in the Part, with their errors.  An infinity or NaN spoils the errors but
+// not the sum, which is then the result.
+template <class Ld_, class PartT>
+struct SumPair : SumF<Ld_, PartT> {
+    using Ld = Ld_;
+    using E = typename Ld::E;
+    using Part = PartT;
+    struct Acc { float s[2], c[2]; };
+    __device__ __forceinline__ static Acc init() { return {{0.f, 0.f}, {0.f, 0.f}}; }
+    __device__ __forceinline__ static void two_sum(float& s, float& c, float v) {
+        const float t = s + v, bp = t - s, ap = t - bp;
+        c = c + ((s - ap) + (v - bp));
+        s = t;
+    }
+    __device__ __forceinline__ static void add(Acc& a, E v, int64_t) { two_sum(a.s[0], a.c[0], v); }
+    template <int K>
+    __device__ __forceinline__ static void add_vec(Acc& a, const E (&e)[K], int64_t) {
+#pragma unroll
+        for (int k = 0; k < K; k++) two_sum(a.s[k & 1], a.c[k & 1], e[k]);
+    }
+    __device__ __forceinline__ static Part to_part(const Acc& a) {
+        float s = a.s[0], c = a.c[0] + a.c[1];
+        two_sum(s, c, a.s[1]);
+        return (Part)s + (Part)(isfinite(c) ? c : 0.f);
+    }
+};
+// FP64_COMBINE: the partials that meet in fp64 are then exact to about 2^-46,
+// however many elements a lane took.  In fp32 a vector cut by a run's end, or a
+// tree of 8, rounded where the kernels before had an element a thread (relative
+// error, fp32 rows of 17 2.6e-8 -> 5.3e-8 -> 2.5e-8, 5000 segments of 23 2.6e-8 ->
+// 4.7e-8 -> 2.5e-8: wide kernels, groups in fp32, this), and adding in double
+// instead is bound by the fp64 pipe.
+template <class Ld_>
+struct GroupTrait<SumF<Ld_, double>> {
+    using type = SumPair<Ld_, double>;
+};
+
 // Compensated sum (Section 1.1, second footnote: Kahan-style compensation).
 // Per thread: kLanes independent fp32 (sum, compensation) pairs, element k of
 // a vector going to lane k mod kLanes (independent dependency chains), each

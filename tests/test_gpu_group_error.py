@@ -47,3 +47,36 @@ def test_fp64_products_round_once(rows, count, each, aux):
                 assert got[r] == np.inf, (r, offset)
             else:
                 assert abs(Fraction(got[r]) - exact) <= bound * exact, (r, offset)
+
+
+@pytest.mark.parametrize("rows,count,each", [(True,) + s for s in ROWS] + [(False,) + s for s in SEGMENTS])
+@pytest.mark.parametrize("dtype", ["f32", "f16", "bf16"])
+def test_fp64_combine_sums_round_once(rows, count, each, dtype):
+    """The result rounds to fp32 once (2^-24 of itself).  Before that only the
+    sum of a lane's rounding errors rounds: with k elements a lane (at most 128
+    here) its j-th addition errs by 2^-24 of at most j 2^-24 of the sum of
+    magnitudes, k^2 2^-49 in all."""
+    import torch
+    x = torch.randn(count * each, generator=torch.Generator().manual_seed(each), dtype=torch.float64)
+    x = x.to(pr.torch_dtype(dtype))
+    want, size = x.view(count, each).double().sum(1).cuda(), x.view(count, each).double().abs().sum(1).cuda()
+    host = x.view(torch.int16).numpy().view(np.uint16) if dtype != "f32" else x.numpy()
+    for offset in (0, 1):
+        got = reduced(host, count, each, dtype, "sum", offset, rows, precision="fp64_combine").double()
+        assert bool(((got - want).abs() <= 2.0 ** -24 * want.abs() + min(each, 128) ** 2 * 2.0 ** -49 * size).all()), offset
+
+
+def test_fp64_combine_infinities_and_nan():
+    """An infinity is the sum, opposite ones and NaN are NaN, wherever they lie."""
+    import torch
+    for each in (23, 200, 4100):
+        x = torch.ones(9, each)
+        x[1, 0] = x[2, -1] = x[3, each // 2] = torch.inf
+        x[4, 1] = -torch.inf
+        x[5, 0], x[5, -1] = torch.inf, -torch.inf
+        x[6, each // 2] = torch.nan
+        for count in (9, 9000):
+            t = x.repeat((count + 8) // 9, 1)[:count]
+            for rows in (True, False):
+                got = reduced(t.numpy().reshape(-1), count, each, "f32", "sum", 1, rows, precision="fp64_combine")
+                assert torch.equal(got.cpu().nan_to_num(-7.0, 8.0, 9.0), t.sum(1).nan_to_num(-7.0, 8.0, 9.0)), (each, count, rows)
