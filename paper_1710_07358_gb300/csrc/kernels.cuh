@@ -673,10 +673,60 @@ __global__ void __launch_bounds__(MaxBlock<T>::value) k_rows(RowArgs a) {
 // Accumulators a lane keeps: one per load in flight where an accumulator is
 // one or two words (shorter chains of dependent operations, and a smaller sum
 // of rounding errors), else one.
-template <class T, int U>
+template <class T, int U, class = void>
 struct GroupAccs {
     static constexpr int value = sizeof(typename T::Acc) <= 8 ? U : 1;
 };
+template <class T, int U>
+struct GroupAccs<T, U, std::void_t<decltype(T::kGroupAccs)>> {
+    static constexpr int value = T::kGroupAccs;
+};
+
+// A trait with a neutral element (pad) takes a vector that a run's end cuts as
+// a whole one, in the order of a tree: added one by one, the elements of such
+// vectors made up most of the rounding error of short runs.
+template <class T, class = void>
+struct HasPad : std::false_type {};
+template <class T>
+struct HasPad<T, std::void_t<decltype(&T::pad)>> : std::true_type {};
+
+// Elements combined as a tree.
+template <class T, int K>
+__device__ __forceinline__ typename T::Part tree(const typename T::Ld::E (&e)[K]) {
+    typename T::Part t[K];
+#pragma unroll
+    for (int k = 0; k < K; k++) t[k] = e[k];
+#pragma unroll
+    for (int s = 1; s < K; s <<= 1)
+#pragma unroll
+        for (int k = 0; k + s < K; k += 2 * s) t[k] = T::combine(t[k], t[k + s]);
+    return t[0];
+}
+
+// Rounds of loads after which a lane's accumulator joins its total: an fp64
+// sum takes no more additions than elements (the fp64 pipe bounds it), but as a
+// tree over a round's vectors and in short chains of those.
+template <class T, class = void>
+struct GroupSteps {
+    static constexpr int value = 0;
+};
+template <class T>
+struct GroupSteps<T, std::void_t<decltype(T::kGroupSteps)>> {
+    static constexpr int value = T::kGroupSteps;
+};
+
+// Accumulators combined as a tree.
+template <class T, int N>
+__device__ __forceinline__ typename T::Part fold_tree(const typename T::Acc (&acc)[N]) {
+    typename T::Part p[N];
+#pragma unroll
+    for (int u = 0; u < N; u++) p[u] = T::to_part(acc[u]);
+#pragma unroll
+    for (int s = 1; s < N; s <<= 1)
+#pragma unroll
+        for (int u = 0; u + s < N; u += 2 * s) p[u] = T::combine(p[u], p[u + s]);
+    return p[0];
+}
 
 // The elements [p0, p0 + len) of x that lane t of G neighbours takes, combined
 // into one Part (the trait is given indices relative to p0, plus i0).  The run is
@@ -701,6 +751,10 @@ __device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In*
     // run-relative element range that whole vectors may be read from
     const int64_t s0 = X0 - p0, s1 = X1 - p0;
     const int c_lo = s0 < -VE ? -VE : (int)s0, c_hi = s1 < (int64_t)len + VE ? (int)s1 : len + VE;
+    constexpr int kSteps = GroupSteps<T>::value;
+    E t_u[U];
+    typename T::Part total = T::part_init();
+    int step = 0;
     for (int j = t; j < nv; j += U * G) {
         Words<kGroupVec> w[U];
 #pragma unroll
@@ -712,12 +766,24 @@ __device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In*
         for (int u = 0; u < U; u++) {
             const int v = j + u * G, c = v * VE - mis;
             typename T::Acc& a = acc[u % NA];
+            if constexpr (kSteps > 0) t_u[u] = T::pad();
             if (v >= nv) continue;
-            if (c >= 0 && c + VE <= len) {
+            const bool whole = c >= 0 && c + VE <= len;
+            if (whole || (HasPad<T>::value && c >= c_lo && c + VE <= c_hi)) {
                 E e[VE];
                 Ld::template dec<kGroupVec>(w[u], e);
-                T::add_vec(a, e, i0 + c);
-            } else if (c >= c_lo && c + VE <= c_hi) {
+                if constexpr (HasPad<T>::value) {
+                    if (!whole) {   // bit k: element c + k belongs to the run
+                        asm volatile("");   // (a branch: selects in every vector cost whole rows a tenth)
+                        const int lo = c < 0 ? -c : 0, hi = len - c < VE ? len - c : VE;
+                        const unsigned m = ((1u << hi) - 1u) >> lo << lo;
+#pragma unroll
+                        for (int k = 0; k < VE; k++) e[k] = m >> k & 1u ? e[k] : T::pad();
+                    }
+                }
+                if constexpr (kSteps > 0) t_u[u] = tree<T>(e);
+                else T::add_vec(a, e, i0 + c);
+            } else if (!HasPad<T>::value && c >= c_lo && c + VE <= c_hi) {
                 E e[VE];
                 Ld::template dec<kGroupVec>(w[u], e);
 #pragma unroll
@@ -728,8 +794,18 @@ __device__ __forceinline__ typename T::Part group_part(const typename T::Ld::In*
                 for (int i = c > 0 ? c : 0; i < e1; i++) T::add(a, Ld::one(x, p0 + i), i0 + i);
             }
         }
+        if constexpr (kSteps > 0) {
+            T::add_tree(acc[0], tree<T>(t_u));
+            if (++step == kSteps) {
+                total = T::combine(total, fold_tree<T, NA>(acc));
+#pragma unroll
+                for (int u = 0; u < NA; u++) acc[u] = T::init();
+                step = 0;
+            }
+        }
     }
-    return fold<T, NA>(acc);
+    if constexpr (kSteps > 0) return T::combine(total, fold_tree<T, NA>(acc));
+    else return fold_tree<T, NA>(acc);
 }
 
 // Combine across the lanes of each group of 2^gl neighbours (gl <= 5; all 32
@@ -807,7 +883,15 @@ __device__ __forceinline__ void warp_segments(const typename T::Ld::In* x, int s
                 // bit i: element c + i belongs to the segment
                 const int lo = c < 0 ? -c : 0, hi = n - c;
                 const unsigned m = (hi >= VE ? (unsigned)((1ull << VE) - 1) : (1u << hi) - 1u) >> lo << lo;
-                if (c >= 0 && hi >= VE) {
+                if constexpr (HasPad<T>::value) {
+                    if (c < 0 || hi < VE) {
+                        asm volatile("");   // (a branch)
+#pragma unroll
+                        for (int q = 0; q < VE; q++) e[q] = m >> q & 1u ? e[q] : T::pad();
+                    }
+                    if constexpr (T::kIdx) T::add_vec(acc, e, c);
+                    else T::add_tree(acc, tree<T>(e));
+                } else if (c >= 0 && hi >= VE) {
                     T::add_vec(acc, e, c);
                 } else {
 #pragma unroll
@@ -829,7 +913,7 @@ __device__ __forceinline__ void warp_segments(const typename T::Ld::In* x, int s
 }
 
 template <class T>
-__global__ void __launch_bounds__(kGroupBlock) k_rows_group(RowGroupArgs a) {
+__device__ __forceinline__ void rows_group_body(const RowGroupArgs& a) {
     using GR = GridR<T>;
     using G = typename GR::Part;
     const auto* x = static_cast<const typename T::Ld::In*>(a.x);
@@ -845,6 +929,31 @@ __global__ void __launch_bounds__(kGroupBlock) k_rows_group(RowGroupArgs a) {
         GR::store(a.out, r, g, false);
         GR::store_aux(a.argidx, a.aux, r, g, 0);
     }
+}
+
+// A trait that declares kGroupBlocks has that many blocks an SM at least (64
+// registers at four: the sums and products of fp32 would take 72, three
+// blocks, [32768, 1000] 24.6 us instead of 22.6).
+template <class T, class = void>
+struct GroupBlocks {
+    static constexpr int value = 0;
+};
+template <class T>
+struct GroupBlocks<T, std::void_t<decltype(T::kGroupBlocks)>> {
+    static constexpr int value = T::kGroupBlocks;
+};
+template <class T>
+__global__ void __launch_bounds__(kGroupBlock) k_rows_group(RowGroupArgs a) {
+    rows_group_body<T>(a);
+}
+template <class T>
+__global__ void __launch_bounds__(kGroupBlock, GroupBlocks<T>::value) k_rows_group_occ(RowGroupArgs a) {
+    rows_group_body<T>(a);
+}
+template <class T>
+constexpr auto rows_group_kernel() {
+    if constexpr (GroupBlocks<T>::value > 0) return &k_rows_group_occ<T>;
+    else return &k_rows_group<T>;
 }
 
 // ------------------------------------------------------------------------
@@ -1306,21 +1415,30 @@ __global__ void __launch_bounds__(kSegBlock, 5) k_seg_group(SegGroupArgs a) {
                     const int len = __shfl_sync(kAll, n0, i);
                     typename T::Acc acc = T::init();
                     int j = t;
+                    // four a step, as a tree where the trait has no index: a
+                    // shorter chain of operations and of roundings
                     for (; j + 3 * lanes < len; j += 4 * lanes) {
                         const typename Ld::E e[4] = {Ld::lone(run[j]), Ld::lone(run[j + lanes]),
                                                      Ld::lone(run[j + 2 * lanes]), Ld::lone(run[j + 3 * lanes])};
-                        // (summed pairwise: a shorter chain of operations and
-                        // of roundings)
-                        if constexpr (!T::kIdx) {
+                        if constexpr (HasPad<T>::value && !T::kIdx) {
+                            T::add_tree(acc, tree<T>(e));
+                        } else if constexpr (!T::kIdx) {
                             T::add_vec(acc, e, 0);
                         } else {
 #pragma unroll
                             for (int q = 0; q < 4; q++) T::add(acc, e[q], j + q * lanes);
                         }
                     }
+                    if constexpr (HasPad<T>::value && !T::kIdx) {
+                        typename Ld::E e[3];
 #pragma unroll
-                    for (int q = 0; q < 3; q++)
-                        if (j + q * lanes < len) T::add(acc, Ld::lone(run[j + q * lanes]), j + q * lanes);
+                        for (int q = 0; q < 3; q++) e[q] = j + q * lanes < len ? Ld::lone(run[j + q * lanes]) : T::pad();
+                        T::add_rest(acc, tree<T>(e));
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 3; q++)
+                            if (j + q * lanes < len) T::add(acc, Ld::lone(run[j + q * lanes]), j + q * lanes);
+                    }
                     const Part p = group_combine<T>(T::to_part(acc), gl);
                     if (t == 0 && len > 0) store_segment<T>(p, s0 + i, a.out, a.argidx, a.aux);
                 }
@@ -1359,7 +1477,7 @@ __global__ void __launch_bounds__(kSegBlock, 5) k_seg_group(SegGroupArgs a) {
 constexpr unsigned kTaskGroup = 64;
 
 template <class T>
-__global__ void __launch_bounds__(kGroupBlock) k_seg_long(SegGroupArgs a) {
+__device__ __forceinline__ void seg_long_body(const SegGroupArgs& a) {
     using Part = typename T::Part;
     constexpr unsigned kAll = 0xffffffffu;
     const auto* x = static_cast<const typename T::Ld::In*>(a.x);
@@ -1452,6 +1570,31 @@ __global__ void __launch_bounds__(kGroupBlock) k_seg_long(SegGroupArgs a) {
             *a.ws.blk_done = 0u;
         }
     }
+}
+
+// A trait that declares kLongBlocks has that many blocks an SM at least (80
+// registers at three: the sums and products of 16-bit types would take 92,
+// two blocks, 8192 segments of 40000 bf16 137 us instead of 120).
+template <class T, class = void>
+struct LongBlocks {
+    static constexpr int value = 0;
+};
+template <class T>
+struct LongBlocks<T, std::void_t<decltype(T::kLongBlocks)>> {
+    static constexpr int value = T::kLongBlocks;
+};
+template <class T>
+__global__ void __launch_bounds__(kGroupBlock) k_seg_long(SegGroupArgs a) {
+    seg_long_body<T>(a);
+}
+template <class T>
+__global__ void __launch_bounds__(kGroupBlock, LongBlocks<T>::value) k_seg_long_occ(SegGroupArgs a) {
+    seg_long_body<T>(a);
+}
+template <class T>
+constexpr auto seg_long_kernel() {
+    if constexpr (LongBlocks<T>::value > 0) return &k_seg_long_occ<T>;
+    else return &k_seg_long<T>;
 }
 
 }  // namespace pr

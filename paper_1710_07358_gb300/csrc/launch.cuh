@@ -38,7 +38,7 @@ cudaError_t launch_seg_long(const SegGroupArgs& a, int grid, int block, cudaStre
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_seg_long<T>, a);
+    cudaLaunchKernelEx(&cfg, seg_long_kernel<T>(), a);
     return cudaGetLastError();
 }
 
@@ -50,7 +50,7 @@ cudaError_t launch_rows(const RowArgs& a, int grid, int block, cudaStream_t st) 
 
 template <class T>
 cudaError_t launch_rows_group(const RowGroupArgs& a, int grid, int block, cudaStream_t st) {
-    k_rows_group<T><<<grid, block, 0, st>>>(a);
+    rows_group_kernel<T>()<<<grid, block, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -132,13 +132,13 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
     if (seg) {
         using G = typename GroupTrait<T>::type;
         reg_add(KernelKey{K_ROWS_GROUP, dtype, op, prec, aux, 0, 0},
-                KernelEntry{reinterpret_cast<const void*>(&k_rows_group<G>),
+                KernelEntry{reinterpret_cast<const void*>(rows_group_kernel<G>()),
                             reinterpret_cast<void*>(&launch_rows_group<G>)});
         KernelEntry sg{reinterpret_cast<const void*>(&k_seg_group<G>), reinterpret_cast<void*>(&launch_seg_group<G>)};
         sg.part_bytes = (int)sizeof(typename G::Part);
         reg_add(KernelKey{K_SEG_GROUP, dtype, op, prec, aux, 0, 0}, sg);
         reg_add(KernelKey{K_SEG_LONG, dtype, op, prec, aux, 0, 0},
-                KernelEntry{reinterpret_cast<const void*>(&k_seg_long<G>),
+                KernelEntry{reinterpret_cast<const void*>(seg_long_kernel<G>()),
                             reinterpret_cast<void*>(&launch_seg_long<G>)});
         reg_axis<T, 2, 0>(dtype, op, prec, aux);
         reg_axis<T, 2, 16>(dtype, op, prec, aux);

@@ -143,6 +143,21 @@ struct GroupTrait {
     using type = T;
 };
 
+// A base that declares kGroupBlocks (k_rows_group) where On.
+template <bool On>
+struct FourBlocks {};
+template <>
+struct FourBlocks<true> {
+    static constexpr int kGroupBlocks = 4;
+};
+// A base that declares kLongBlocks (k_seg_long) where On.
+template <bool On>
+struct LongThree {};
+template <>
+struct LongThree<true> {
+    static constexpr int kLongBlocks = 3;
+};
+
 // Output writers for float-valued results.
 __device__ __forceinline__ void put_f32(void* out, int64_t i, float v) { static_cast<float*>(out)[i] = v; }
 __device__ __forceinline__ void put_f64(void* out, int64_t i, double v) { static_cast<double*>(out)[i] = v; }
@@ -192,7 +207,7 @@ struct SumF {
 // in the Part, with their errors.  An infinity or NaN spoils the errors but
 // not the sum, which is then the result.
 template <class Ld_, class PartT>
-struct SumPair : SumF<Ld_, PartT> {
+struct SumPair : SumF<Ld_, PartT>, FourBlocks<Ld_::ES == 2> {
     using Ld = Ld_;
     using E = typename Ld::E;
     using Part = PartT;
@@ -224,6 +239,48 @@ struct SumPair : SumF<Ld_, PartT> {
 template <class Ld_>
 struct GroupTrait<SumF<Ld_, double>> {
     using type = SumPair<Ld_, double>;
+};
+
+// PLAIN: trees of up to eight elements join a lane's sum with the rounding
+// error kept, so that a lane's error does not grow with the elements it takes.
+// The error is Dekker's, which is exact when the sum is the larger of the two
+// and otherwise off by no more than the rounding it stands for: four operations
+// a tree instead of TwoSum's seven.
+template <class Ld_>
+struct SumTree : SumF<Ld_, float>, FourBlocks<Ld_::ES == 4>, LongThree<Ld_::ES == 2> {
+    using Ld = Ld_;
+    using E = typename Ld::E;
+    using Part = float;
+    struct Acc { float s, c; };
+    static constexpr int kGroupAccs = 1;
+    __device__ __forceinline__ static Acc init() { return {0.f, 0.f}; }
+    __device__ __forceinline__ static E pad() { return 0.f; }
+    __device__ __forceinline__ static void add_tree(Acc& a, float v) {
+        const float t = a.s + v;
+        a.c = a.c + (v - (t - a.s));
+        a.s = t;
+    }
+    // (the last few of a short run: one rounding a lane)
+    __device__ __forceinline__ static void add_rest(Acc& a, float v) { a.s = a.s + v; }
+    __device__ __forceinline__ static void add(Acc& a, E v, int64_t) { add_tree(a, v); }
+    template <int K>
+    __device__ __forceinline__ static void add_vec(Acc& a, const E (&e)[K], int64_t) {
+        constexpr int N = K < 8 ? K : 8;
+#pragma unroll
+        for (int h = 0; h < K; h += N) {
+            float t = 0.f;   // SumF's tree of N elements
+            float v[N];
+#pragma unroll
+            for (int k = 0; k < N; k++) v[k] = e[h + k];
+            SumF<Ld_, float>::add_vec(t, v, 0);
+            add_tree(a, t);
+        }
+    }
+    __device__ __forceinline__ static Part to_part(const Acc& a) { return a.s + (isfinite(a.c) ? a.c : 0.f); }
+};
+template <class Ld_>
+struct GroupTrait<SumF<Ld_, float>> {
+    using type = SumTree<Ld_>;
 };
 
 // Compensated sum (Section 1.1, second footnote: Kahan-style compensation).
@@ -315,7 +372,12 @@ struct SumF64 {
     using Acc = double;
     using Part = double;
     static constexpr bool kIdx = false;
+    static constexpr int kGroupAccs = 1;    // (groups of lanes: see group_part)
+    static constexpr int kGroupSteps = 4;
     __device__ __forceinline__ static Acc init() { return 0.0; }
+    __device__ __forceinline__ static E pad() { return 0.0; }
+    __device__ __forceinline__ static void add_tree(Acc& a, E v) { a = a + v; }
+    __device__ __forceinline__ static void add_rest(Acc& a, E v) { a = a + v; }
     template <int K>
     __device__ __forceinline__ static void add_vec(Acc& a, const E (&e)[K], int64_t) {
         double t[K];
@@ -778,6 +840,44 @@ struct ProdF {
     }
 };
 
+// The product's group form: pairs of factors, each joined to the lane's product
+// with its rounding error kept (TwoProduct by fma).  Factors near one, as the
+// gradients meet them, round with a bias, and by an amount that depends on the
+// order: a lane's error is that of its pairs, half of its roundings, however
+// many factors it takes.  The error is left out where it says nothing: zeros,
+// infinities, NaN.
+template <class Ld_>
+struct ProdTree : ProdF<Ld_>, FourBlocks<Ld_::ES == 4>, LongThree<Ld_::ES == 2> {
+    using Ld = Ld_;
+    using E = typename Ld::E;
+    using Part = float;
+    struct Acc { float p, c; };
+    static constexpr int kGroupAccs = 1;
+    __device__ __forceinline__ static Acc init() { return {1.f, 0.f}; }
+    __device__ __forceinline__ static E pad() { return 1.f; }
+    __device__ __forceinline__ static void add(Acc& a, E v, int64_t) {
+        const float t = a.p * v;
+        a.c = __fmaf_rn(a.c, v, __fmaf_rn(a.p, v, -t));
+        a.p = t;
+    }
+    template <int K>
+    __device__ __forceinline__ static void add_vec(Acc& a, const E (&e)[K], int64_t i) {
+        static_assert(K % 2 == 0, "pairs");
+#pragma unroll
+        for (int k = 0; k < K; k += 2) add(a, e[k] * e[k + 1], i);
+    }
+    // (short runs, which take nothing else: their order is a tree's anyway)
+    __device__ __forceinline__ static void add_tree(Acc& a, E v) { a.p = a.p * v; }
+    __device__ __forceinline__ static void add_rest(Acc& a, E v) { a.p = a.p * v; }
+    __device__ __forceinline__ static Part to_part(const Acc& a) {
+        return a.p != 0.f && isfinite(a.c) ? a.p + a.c : a.p;
+    }
+};
+template <class Ld_>
+struct GroupTrait<ProdF<Ld_>> {
+    using type = ProdTree<Ld_>;
+};
+
 // fp64 product on the integer pipes.  GB300's fp64 units issue ~0.5e12
 // multiplies/s, slower than HBM delivers doubles (~0.9e12/s), so the combine
 // keeps a 64-bit significand m in [2^63, 2^64) and a 64-bit exponent e
@@ -980,6 +1080,11 @@ struct ProdAux {
         store(out, i, e, f64);
         store_aux(nullptr, aux, i, e, 0);
     }
+};
+
+template <class Base>
+struct GroupTrait<ProdAux<Base>> {
+    using type = ProdAux<typename GroupTrait<Base>::type>;
 };
 
 }  // namespace pr

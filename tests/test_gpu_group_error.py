@@ -80,3 +80,90 @@ def test_fp64_combine_infinities_and_nan():
             for rows in (True, False):
                 got = reduced(t.numpy().reshape(-1), count, each, "f32", "sum", 1, rows, precision="fp64_combine")
                 assert torch.equal(got.cpu().nan_to_num(-7.0, 8.0, 9.0), t.sum(1).nan_to_num(-7.0, 8.0, 9.0)), (each, count, rows)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("each,levels", [(17, 4), (33, 6)])
+def test_sums_beside_one_large_element(dtype, each, levels):
+    """Each small element is half a unit in the last place of the large one, so
+    every addition to it may lose one.  A vector is a tree of at most eight
+    (three roundings), the lane's sum keeps what it loses, its result rounds
+    once, and at most four lanes combine (two levels)."""
+    count = 200000
+    big, small = 2.0 ** 15, 2.0 ** -9
+    x = np.full((count, each), small, np.float32)
+    x[np.arange(count), np.arange(count) % each] = big
+    host = x.astype(np.float16) if dtype == "f16" else (x.view(np.uint32) >> 16).astype(np.uint16) if dtype == "bf16" else x
+    want = big + (each - 1) * small
+    for offset in (0, 1, 5):
+        got = reduced(host.reshape(-1), count, each, dtype, "sum", offset, True).double().cpu().numpy()
+        assert np.abs(got - want).max() <= levels * small, offset
+
+
+def test_fp64_long_segments_beside_one_large_element():
+    """Vectors of the small elements are half a unit in the last place of the
+    large one: a lane's chain may lose one a step, and blocks of four steps
+    end each chain.  Lost at most: the large element's own vector (1), its
+    block's other steps (3), and what the chunk's cut vectors and last block
+    add up to (6)."""
+    import torch
+    nseg, each = 8200, 16384
+    n = np.ones(nseg, np.int64)
+    long = np.arange(5, nseg, 410)
+    n[long] = each
+    off = np.concatenate([[0], np.cumsum(n)])
+    x = np.full(int(off[-1]), 0.5)
+    for k, s in enumerate(long):
+        x[off[s] + (k * 761) % each] = 2.0 ** 54
+    got = pr.segmented_reduce(torch.from_numpy(x).cuda(), torch.from_numpy(off).cuda(), "sum").cpu().numpy()
+    assert np.abs(got[long] - 2.0 ** 54 - (each - 1) / 2).max() <= 10 * 2
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("aux", [False, True])
+def test_products_of_factors_near_one(dtype, aux):
+    """Trees of four and exact joins: three of four factors round (2^-24 each,
+    with aux none but the joins), and 64 more cover the lanes', warps' and
+    final roundings; the bound without them, n - 1 roundings, is what any
+    order gives."""
+    import torch
+    if aux and dtype != "f32":
+        pytest.skip("the gradient's state exists for f32 and f64")
+    for rows, count, each in [(True,) + s for s in ROWS] + [(False,) + s for s in SEGMENTS]:
+        x = 1 + torch.randn(count * each, generator=torch.Generator().manual_seed(each)) * (0.3 / each ** 0.5)
+        x = x.to(pr.torch_dtype(dtype))
+        want = x.double().view(count, each).prod(1).cuda()
+        host = x.view(torch.int16).numpy().view(np.uint16) if dtype != "f32" else x.numpy()
+        got = reduced(host, count, each, dtype, "prod", 1, rows, aux=aux).double()
+        assert bool(((got - want).abs() <= (0.75 * each + 64) * 2.0 ** -24 * want.abs()).all()), (rows, count, each)
+
+
+@pytest.mark.parametrize("op", ["sum", "prod"])
+def test_special_values_in_trees(op):
+    """Infinities, NaN, zeros of both signs and overflow, wherever they lie."""
+    import torch
+    for each in (3, 23, 200, 4100):
+        x = torch.ones(12, each)
+        x[1, 0] = x[2, -1] = x[3, each // 2] = torch.inf
+        x[4, 1] = -torch.inf
+        x[5, 0], x[5, -1] = torch.inf, -torch.inf
+        x[6, each // 2] = torch.nan
+        x[7, 1], x[7, 2] = 0.0, torch.inf
+        x[8, each // 2] = -0.0
+        x[9] = -0.0
+        x[10, :3] = 3e38
+        x[11, 0] = 1e-30
+        x[11, 1] = 1e-30
+        want = torch.stack([getattr(torch, op)(r) for r in x]) if op == "sum" else x.double().prod(1).float()
+        for count in (12, 9000):
+            t = x.repeat((count + 11) // 12, 1)[:count]
+            w = want.repeat((count + 11) // 12)[:count]
+            for rows in (True, False):
+                got = reduced(t.numpy().reshape(-1), count, each, "f32", op, 1, rows).cpu()
+                keep = torch.arange(count) % 12 != (10 if op == "sum" else 99)   # (order decides that sum's overflow)
+                same = (got == w) | (got.isnan() & w.isnan())
+                if op == "sum":
+                    same |= (got - w).abs() <= each * 2.0 ** -24 * w.abs()
+                assert bool(same[keep].all()), (each, count, rows, got[:12], w[:12])
+                if op == "prod":
+                    assert torch.equal(torch.signbit(got[w == 0]), torch.signbit(w[w == 0])), (each, count, rows)
