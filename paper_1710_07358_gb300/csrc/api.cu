@@ -797,6 +797,11 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
     if (splits > 1024) splits = 1024;
     if (splits > 1 && vb == 32 && stream_us > 1.0 && part * splits > 0.05) {
         // the warps of a block share a tile's rows, then blocks split them
+        // (plain sums of 16-bit types pass fp64 partials on: short rows of them
+        // add up exactly in fp32, and the fewer, longer partials of shared
+        // splits would each round; [16, 4096, 512] fp16 error 5.5e-8 with
+        // splits of a warp, 8.7e-8 with fp32 partials, 2.5e-8 with these)
+        if (op == PR_SUM && prec == PR_PREC_PLAIN && es == 2) prec = PR_PREC_FP64_COMBINE;
         const KernelEntry* ec = reg_find(KernelKey{K_AXIS_COOP, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux, 2, 32});
         if (!ec) return fail(PR_ERR_UNSUPPORTED, "no axis kernel for dtype %d op %d precision %d", dtype, op, prec);
         e = ec;
@@ -806,7 +811,7 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
         s = occupancy(e->fn, c.block, &occ);
         if (s != PR_OK) return s;
         if (occ < 1) return fail(PR_ERR_UNSUPPORTED, "axis kernel cannot run with %d threads per block", c.block);
-        splits = axis_splits(tiles, (int64_t)di.sms * occ, most / a.coop, stream_us, part);
+        splits = axis_splits(tiles, (int64_t)di.sms * occ, most / a.coop, stream_us, 2.0 * e->part_bytes / ((double)n * es));
     }
     a.splits = splits;
     // a warp holds fewer than 2^31 rows (the float arg-extremum keeps its

@@ -12,15 +12,19 @@
 //   U rows' loads before accumulating any of them.  The lanes that share a
 //   column then combine by an xor butterfly over the row bits of the lane
 //   index, in a fixed order.  Where tiles alone leave warps idle, the warps of
-//   a block share a tile's rows first and combine through shared memory (in
-//   warp order), and only then are the rows split over blocks: a partial per
+//   a block share a tile's rows first and combine through shared memory (as a
+//   tree), and only then are the rows split over blocks: a partial per
 //   warp and output cost more traffic than the input where the axis is short
 //   ([64, 577, 768] fp32 maximum with index: 49 splits wrote and read 38 MB
-//   each of 16-byte partials for 113 MB of input; with shared splits 77 -> 31
-//   us, 0.54 of a 6.8 TB/s copy: one wave of blocks, bound by latency).  With one split the outputs
-//   are written; with more, the partials, and k_axis_finish combines each output's
-//   partials in a fixed order (one thread per output folding the splits in
-//   order, or with many splits one warp per output and a fixed tree), so
+//   each of 16-byte partials for 113 MB of input; with shared splits 77 -> 27
+//   us, 0.62 of a 6.8 TB/s copy: one wave of blocks, bound by latency).  A lane
+//   then takes more rows of a column than a split's lane did, so sums and
+//   products take the AxisTrait form, which keeps what they round off (error
+//   of the fp32 sum of [1, 5000, 4096] 1.2e-7 with splits of a warp, 1.5e-7 by
+//   plain chains, 7.8e-8 now; fp64 2.1e-16, 2.8e-16, 2.0e-16).  With one split
+//   the outputs are written; with more, the partials, and k_axis_finish combines each output's
+//   partials in a fixed order (one thread per output folding the splits as
+//   trees of eight, or with many splits one warp per output and a fixed tree), so
 //   results are deterministic for a fixed launch shape.
 // k_axis_backward  gradient of an axis reduction: grad_in[p, i, q] from
 //   grad_out[p, q] and the per-output state, one streaming write.
@@ -72,11 +76,28 @@ __device__ __forceinline__ void add_in_order(typename T::Acc& a, typename T::Ld:
     else T::add(a, v, i);
 }
 
+// What the warps that share a split exchange: Parts, or a trait's accumulators
+// where it can merge them (no rounding lost, and no fp64 operation a warp).
+template <class T, class = void>
+struct ColPart {
+    using P = typename T::Part;
+    __device__ __forceinline__ static P from(const typename T::Acc& a) { return T::to_part(a); }
+    __device__ __forceinline__ static P combine(const P& a, const P& b) { return T::combine(a, b); }
+    __device__ __forceinline__ static typename T::Part part(const P& p) { return p; }
+};
+template <class T>
+struct ColPart<T, std::void_t<decltype(&T::merge)>> {
+    using P = typename T::Acc;
+    __device__ __forceinline__ static P from(const typename T::Acc& a) { return a; }
+    __device__ __forceinline__ static P combine(const P& a, const P& b) { return T::merge(a, b); }
+    __device__ __forceinline__ static typename T::Part part(const P& p) { return T::to_part(p); }
+};
+
 // Column elements (a divisor of VE) whose partials of kAxisCoop warps meet in
 // shared memory at a time: up to 16 KB.
 template <class T, int VE>
 struct AxisPhase {
-    static constexpr int kBytes = kAxisCoop * 32 * (int)sizeof(typename T::Part);
+    static constexpr int kBytes = kAxisCoop * 32 * (int)sizeof(typename ColPart<T>::P);
     static constexpr int fit(int k) { return k > 1 && k * kBytes > 16384 ? fit(k / 2) : k; }
     static constexpr int value = fit(VE);
 };
@@ -124,14 +145,8 @@ __global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_
     const int64_t slab = p * a.n * a.inner + col * VE;  // element offset of (p, row 0, this column)
 
     Acc acc[VE];
-    constexpr bool kBlocked = COOP && !Exact<T>::value && sizeof(Acc) == 4 && VE * sizeof(Part) <= 64;   // (registers)
-    constexpr int kBlockSteps = sizeof(Part) == 8 ? 8 : 4;   // (fp64 additions are slow)
-    Part total[kBlocked ? VE : 1];
 #pragma unroll
-    for (int k = 0; k < VE; k++) {
-        acc[k] = T::init();
-        if constexpr (kBlocked) total[k] = T::part_init();
-    }
+    for (int k = 0; k < VE; k++) acc[k] = T::init();
     if constexpr (HasOrderedPair<T>::value) {
         // per element the running extremum and its row relative to r0 (a
         // split holds fewer than 2^31 rows): three operations an element
@@ -183,24 +198,20 @@ __global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_
         }
     } else if (has) {
         int64_t r = r0 + ty;
-        // an inexact 32-bit accumulator joins its Part every kBlockSteps
-        // steps: a shorter chain of roundings, whatever the split
-        if constexpr (kBlocked) {
-            for (; r + (int64_t)(kBlockSteps * U - 1) * ry < r1;) {
-#pragma unroll 1
-                for (int b = 0; b < kBlockSteps; b++, r += (int64_t)U * ry) {
-                    E e[U][VE];
+        // sums and products take the rows of a step as a tree (an fp64 sum
+        // four: a shorter chain for the same additions)
+        if constexpr (COOP && HasPad<T>::value && !T::kIdx) {
+            constexpr int R = sizeof(E) == 8 ? 4 : U;
+            for (; r + (int64_t)(R - 1) * ry < r1; r += (int64_t)R * ry) {
+                E e[R][VE];
 #pragma unroll
-                    for (int u = 0; u < U; u++) axis_load<VB, Ld>(x, slab + (r + (int64_t)u * ry) * a.inner, e[u]);
-#pragma unroll
-                    for (int u = 0; u < U; u++)
-#pragma unroll
-                        for (int k = 0; k < VE; k++) add_in_order<T>(acc[k], e[u][k], r + (int64_t)u * ry);
-                }
+                for (int u = 0; u < R; u++) axis_load<VB, Ld>(x, slab + (r + (int64_t)u * ry) * a.inner, e[u]);
 #pragma unroll
                 for (int k = 0; k < VE; k++) {
-                    total[k] = T::combine(total[k], T::to_part(acc[k]));
-                    acc[k] = T::init();
+                    E t[R];
+#pragma unroll
+                    for (int u = 0; u < R; u++) t[u] = e[u][k];
+                    T::add_vec(acc[k], t, r);
                 }
             }
         }
@@ -234,24 +245,28 @@ __global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_
         }
     };
     // a warp's column elements combine across its rows' lanes; then (COOP),
-    // KP elements at a time, across the block's warps in warp order, each
-    // element by one of the warps
+    // KP elements at a time, across the block's warps as a tree, each element
+    // by one of the warps
     if constexpr (COOP) {
         constexpr int KP = AxisPhase<T, VE>::value;
-        __shared__ Part s_part[KP][kAxisCoop][32];
+        using CP = ColPart<T>;
+        using P = typename CP::P;
+        __shared__ P s_part[KP][kAxisCoop][32];
         const int warp = threadIdx.x >> 5;
 #pragma unroll
         for (int k = 0; k < VE; k++) {
-            Part q = T::to_part(acc[k]);
-            if constexpr (kBlocked) q = T::combine(total[k], q);
-            for (int m = 16; m >= bx; m >>= 1) q = T::combine(q, shfl_xor_any(q, m));
+            P q = CP::from(acc[k]);
+            for (int m = 16; m >= bx; m >>= 1) q = CP::combine(q, shfl_xor_any(q, m));
             s_part[k % KP][warp][lane] = q;
             if (k % KP == KP - 1) {
                 __syncthreads();
                 for (int j = warp; j < KP; j += a.coop) {
-                    q = s_part[j][0][lane];
-                    for (int w = 1; w < a.coop; w++) q = T::combine(q, s_part[j][w][lane]);
-                    result(k - (KP - 1) + j, q);
+                    // as a tree: coop is a power of two of at most eight
+                    auto pair = [&](int w) { return CP::combine(s_part[j][w][lane], s_part[j][w + 1][lane]); };
+                    auto quad = [&](int w) { return CP::combine(pair(w), pair(w + 2)); };
+                    q = a.coop == 8 ? CP::combine(quad(0), quad(4))
+                                    : (a.coop == 4 ? quad(0) : (a.coop == 2 ? pair(0) : s_part[j][0][lane]));
+                    result(k - (KP - 1) + j, CP::part(q));
                 }
                 if (k < VE - 1) __syncthreads();   // before the slots are written again
             }
@@ -266,7 +281,7 @@ __global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_
     }
 }
 
-// Few splits: one thread per output folds its splits in order.  Many: one
+// Few splits: one thread per output folds its splits in order, as trees of eight.  Many: one
 // warp per output, the lanes taking the splits in order (lane, lane + 32, ...)
 // and combining by a fixed butterfly.
 template <class T>
@@ -279,8 +294,12 @@ __global__ void __launch_bounds__(256) k_axis_finish(AxisArgs a) {
     if (a.splits <= kAxisThreadFinish) {
         const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
         if (o >= nout) return;
-        G q = part[o];
-        for (int64_t s = 1; s < a.splits; s++) q = GR::combine(q, part[s * nout + o]);
+        auto at = [&](int64_t s) { return s < a.splits ? part[s * nout + o] : GR::part_init(); };
+        auto pair = [&](int64_t s) { return GR::combine(at(s), at(s + 1)); };
+        auto quad = [&](int64_t s) { return GR::combine(pair(s), pair(s + 2)); };
+        auto eight = [&](int64_t s) { return s + 4 < a.splits ? GR::combine(quad(s), quad(s + 4)) : quad(s); };
+        G q = eight(0);
+        for (int64_t s = 8; s < a.splits; s += 8) q = GR::combine(q, eight(s));
         GR::store(a.out, o, q, a.out_f64 != 0);
         GR::store_aux(a.argidx, a.aux, o, q, 0);
         return;

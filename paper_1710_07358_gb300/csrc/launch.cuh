@@ -146,7 +146,7 @@ void reg_family(uint8_t dtype, uint8_t op, uint8_t prec, uint8_t aux, bool plain
         reg_axis<T, 4, 0>(dtype, op, prec, aux);
         reg_axis<T, 4, 16>(dtype, op, prec, aux);
         reg_axis<T, 4, 32>(dtype, op, prec, aux);
-        reg_axis<T, 2, 32, true>(dtype, op, prec, aux);
+        reg_axis<typename AxisTrait<T>::type, 2, 32, true>(dtype, op, prec, aux);
         reg_add(KernelKey{K_AXIS_FINISH, dtype, op, prec, aux, 0, 0},
                 KernelEntry{reinterpret_cast<const void*>(&k_axis_finish<T>),
                             reinterpret_cast<void*>(&launch_axis_finish<T>)});

@@ -143,6 +143,13 @@ struct GroupTrait {
     using type = T;
 };
 
+// The trait of the axis kernel whose blocks' warps share a split: as there, a
+// lane takes more elements of a column than a lane of the splits before did.
+template <class T>
+struct AxisTrait {
+    using type = T;
+};
+
 // A base that declares kGroupBlocks (k_rows_group) where On.
 template <bool On>
 struct FourBlocks {};
@@ -246,11 +253,11 @@ struct GroupTrait<SumF<Ld_, double>> {
 // The error is Dekker's, which is exact when the sum is the larger of the two
 // and otherwise off by no more than the rounding it stands for: four operations
 // a tree instead of TwoSum's seven.
-template <class Ld_>
-struct SumTree : SumF<Ld_, float>, FourBlocks<Ld_::ES == 4>, LongThree<Ld_::ES == 2> {
+template <class Ld_, class PartT>
+struct SumTree : SumF<Ld_, PartT>, FourBlocks<Ld_::ES == 4>, LongThree<Ld_::ES == 2> {
     using Ld = Ld_;
     using E = typename Ld::E;
-    using Part = float;
+    using Part = PartT;
     struct Acc { float s, c; };
     static constexpr int kGroupAccs = 1;
     __device__ __forceinline__ static Acc init() { return {0.f, 0.f}; }
@@ -259,6 +266,14 @@ struct SumTree : SumF<Ld_, float>, FourBlocks<Ld_::ES == 4>, LongThree<Ld_::ES =
         const float t = a.s + v;
         a.c = a.c + (v - (t - a.s));
         a.s = t;
+    }
+    // two lanes' sums, errors and all (TwoSum): what lanes and warps exchange
+    // where they share a column, on the fp32 pipe
+    __device__ __forceinline__ static Acc merge(const Acc& a, const Acc& b) {
+        Acc r = a;
+        SumPair<Ld_, float>::two_sum(r.s, r.c, b.s);
+        r.c = r.c + b.c;
+        return r;
     }
     // (the last few of a short run: one rounding a lane)
     __device__ __forceinline__ static void add_rest(Acc& a, float v) { a.s = a.s + v; }
@@ -272,15 +287,15 @@ struct SumTree : SumF<Ld_, float>, FourBlocks<Ld_::ES == 4>, LongThree<Ld_::ES =
             float v[N];
 #pragma unroll
             for (int k = 0; k < N; k++) v[k] = e[h + k];
-            SumF<Ld_, float>::add_vec(t, v, 0);
+            SumF<Ld_, PartT>::add_vec(t, v, 0);
             add_tree(a, t);
         }
     }
-    __device__ __forceinline__ static Part to_part(const Acc& a) { return a.s + (isfinite(a.c) ? a.c : 0.f); }
+    __device__ __forceinline__ static Part to_part(const Acc& a) { return (Part)a.s + (Part)(isfinite(a.c) ? a.c : 0.f); }
 };
 template <class Ld_>
 struct GroupTrait<SumF<Ld_, float>> {
-    using type = SumTree<Ld_>;
+    using type = SumTree<Ld_, float>;
 };
 
 // Compensated sum (Section 1.1, second footnote: Kahan-style compensation).
@@ -875,6 +890,14 @@ struct ProdTree : ProdF<Ld_>, FourBlocks<Ld_::ES == 4>, LongThree<Ld_::ES == 2> 
 };
 template <class Ld_>
 struct GroupTrait<ProdF<Ld_>> {
+    using type = ProdTree<Ld_>;
+};
+template <class Ld_, class PartT>
+struct AxisTrait<SumF<Ld_, PartT>> {
+    using type = SumTree<Ld_, PartT>;
+};
+template <class Ld_>
+struct AxisTrait<ProdF<Ld_>> {
     using type = ProdTree<Ld_>;
 };
 
