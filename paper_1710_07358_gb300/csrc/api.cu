@@ -605,22 +605,28 @@ static int rows_group_lanes(int64_t rows, int64_t nv, int es, int sms) {
     return gl;
 }
 
+// Lanes per row (log2) of the row kernel by groups, or -1: the call takes the
+// other kernels.
+static int rows_by_groups(const void* x, int64_t rows, int64_t cols, int dtype, int sms) {
+    const int es = elem_size(dtype);
+    const uintptr_t mis = reinterpret_cast<uintptr_t>(x) % kGroupVec;
+    if (rows < 1 || rows > (int64_t)1 << 50 || cols < 1 || mis % es) return -1;
+    // whole vectors, or one more where rows start off the vector grid
+    const int64_t ve = kGroupVec / es;
+    const int64_t nv = cols % ve == 0 && mis == 0 ? cols / ve : cols / ve + 2;
+    return rows_group_lanes(rows, nv, es, sms);
+}
+
 // Rows by groups of lanes (any length and alignment); PR_ERR_UNSUPPORTED
 // (nothing enqueued, no message kept) when they are left to the other kernels.
 static pr_status run_rows_group(const void* x, int64_t rows, int64_t cols, int dtype, int op, int prec, int aux,
                                 void* out, int64_t* argidx, pr_prod_aux* paux, cudaStream_t st) {
-    const int es = elem_size(dtype);
-    const uintptr_t mis = reinterpret_cast<uintptr_t>(x) % kGroupVec;
-    if (rows < 1 || rows > (int64_t)1 << 50 || cols < 1 || mis % es) return PR_ERR_UNSUPPORTED;
     const KernelEntry* e = reg_find(KernelKey{K_ROWS_GROUP, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux, 0, 0});
     if (!e) return PR_ERR_UNSUPPORTED;
     DevInfo di;
     pr_status s = device_info(&di, nullptr);
     if (s != PR_OK) return s;
-    // whole vectors, or one more where rows start off the vector grid
-    const int64_t ve = kGroupVec / es;
-    const int64_t nv = cols % ve == 0 && mis == 0 ? cols / ve : cols / ve + 2;
-    const int gl = rows_group_lanes(rows, nv, es, di.sms);
+    const int gl = rows_by_groups(x, rows, cols, dtype, di.sms);
     if (gl < 0) return PR_ERR_UNSUPPORTED;
     const int64_t grid = ((rows << gl) + kGroupBlock - 1) / kGroupBlock;
     if (grid > 0x7fffffff) return PR_ERR_UNSUPPORTED;
@@ -630,7 +636,8 @@ static pr_status run_rows_group(const void* x, int64_t rows, int64_t cols, int d
     Workspace ws;
     s = get_ws(st, &ws);
     if (s != PR_OK) return s;
-    RowGroupArgs a{x, rows, cols, (int)mis / es, gl, out, argidx, paux};
+    const int shift = (int)(reinterpret_cast<uintptr_t>(x) % kGroupVec) / elem_size(dtype);
+    RowGroupArgs a{x, rows, cols, shift, gl, out, argidx, paux};
     PR_INJECT_LAUNCH();
     cudaError_t err = reinterpret_cast<RowGroupLaunch>(e->launch)(a, (int)grid, kGroupBlock, st);
     if (err != cudaSuccess) return fail(PR_ERR_CUDA, "row launch: %s", cudaGetErrorString(err));
@@ -738,39 +745,33 @@ static int64_t axis_splits(int64_t tiles, int64_t resident, int64_t most, double
     return best;
 }
 
-// Reduction of the middle axis of [outer, n, inner] (inner > 1, outer > 0).
-// The launch: a warp per (slab, column group), times row splits where those do
+struct AxisPlan {
+    const KernelEntry* e = nullptr;
+    int prec;            // of the kernels that run
+    int block;
+    bool shared = false; // the warps of a block share a split
+};
+
+// The launch of a reduction of the middle axis of [outer, n, inner] (inner > 1,
+// outer and n > 0; a.x and the sizes given): a warp per (slab, column group), times row splits where those do
 // not fill the GPU twice.  Splits of a warp each leave a partial each; where
 // those come to more than a twentieth of the input's traffic, the warps of a
 // block share a split instead, and axis_splits has their number (measured on
 // GB300, us: [64, 577, 768] fp32 maximum with index 77 with 49 splits of a
-// warp, 31 shared; [4096, 16, 512] sum 44 and 32; [16, 4096, 4096] sum 159 and
+// warp, 27 shared; [4096, 16, 512] sum 44 and 33; [16, 4096, 4096] sum 159 and
 // 166, maximum 168 and 199).  Inputs below 7 MB are bound by latency either
 // way, and columns that are not whole vectors keep more rows in flight in the
 // smaller kernel ([1, 5000, 4099] maximum 49 and 57).  splits > 1 add a
 // finishing pass.
-static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner, int dtype, int op, int prec,
-                          int aux, void* out, int64_t* argidx, pr_prod_aux* paux, cudaStream_t st,
-                          const pr_config& cfg) {
+static pr_status axis_plan(AxisArgs& a, int dtype, int op, int prec, int aux, const pr_config& cfg, AxisPlan* plan) {
+    const int64_t outer = a.outer, n = a.n, inner = a.inner;
     const int es = elem_size(dtype);
     DevInfo di;
     pr_status s = device_info(&di, nullptr);
     if (s != PR_OK) return s;
-    AxisArgs a{x, outer, n, inner, 0, 1, 0, 1, 1, 0, out, argidx, paux, 0, nullptr};
-    if (n == 0) {
-        const KernelEntry* e = reg_find(KernelKey{K_AXIS_EMPTY, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec,
-                                                  (uint8_t)aux, 0, 0});
-        if (!e) return fail(PR_ERR_UNSUPPORTED, "no axis kernel for dtype %d op %d precision %d", dtype, op, prec);
-        const int64_t nout = outer * inner;
-        int grid = (int)((nout + 255) / 256 < 4096 ? (nout + 255) / 256 : 4096);
-        PR_INJECT_LAUNCH();
-        cudaError_t err = reinterpret_cast<AxisLaunch>(e->launch)(a, grid, 256, st);
-        if (err != cudaSuccess) return fail(PR_ERR_CUDA, "axis launch: %s", cudaGetErrorString(err));
-        return PR_OK;
-    }
     // vector columns when a row is a whole number of aligned vectors, else one element per lane
     int vb = cfg.vec_bytes;
-    if (inner % (vb / es) != 0 || reinterpret_cast<uintptr_t>(x) % (uintptr_t)vb != 0) vb = 0;
+    if (inner % (vb / es) != 0 || reinterpret_cast<uintptr_t>(a.x) % (uintptr_t)vb != 0) vb = 0;
     const KernelEntry* e = reg_find(KernelKey{K_AXIS, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux,
                                               (uint8_t)cfg.unroll, (uint8_t)vb});
     if (!e) return fail(PR_ERR_UNSUPPORTED, "no axis kernel for dtype %d op %d precision %d", dtype, op, prec);
@@ -805,6 +806,7 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
         const KernelEntry* ec = reg_find(KernelKey{K_AXIS_COOP, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec, (uint8_t)aux, 2, 32});
         if (!ec) return fail(PR_ERR_UNSUPPORTED, "no axis kernel for dtype %d op %d precision %d", dtype, op, prec);
         e = ec;
+        plan->shared = true;
         const int64_t most = n / (32 / bx * 2 * 4) > 1 ? n / (32 / bx * 2 * 4) : 1;
         while (a.coop < kAxisCoop && 2 * a.coop <= most) a.coop *= 2;
         c.block = 32 * a.coop;
@@ -822,6 +824,32 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
     a.rows_per_split = (n + a.splits * a.coop - 1) / (a.splits * a.coop);
     // (splits past the last row would leave partials of no rows: identities)
     a.splits = (n + a.rows_per_split * a.coop - 1) / (a.rows_per_split * a.coop);
+    plan->e = e;
+    plan->prec = prec;
+    plan->block = c.block;
+    return PR_OK;
+}
+
+// Reduction of the middle axis of [outer, n, inner] (inner > 1, outer > 0).
+static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner, int dtype, int op, int prec,
+                          int aux, void* out, int64_t* argidx, pr_prod_aux* paux, cudaStream_t st,
+                          const pr_config& cfg) {
+    AxisArgs a{x, outer, n, inner, 0, 1, 0, 1, 1, 0, out, argidx, paux, 0, nullptr};
+    if (n == 0) {
+        const KernelEntry* e = reg_find(KernelKey{K_AXIS_EMPTY, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec,
+                                                  (uint8_t)aux, 0, 0});
+        if (!e) return fail(PR_ERR_UNSUPPORTED, "no axis kernel for dtype %d op %d precision %d", dtype, op, prec);
+        const int64_t nout = outer * inner;
+        int grid = (int)((nout + 255) / 256 < 4096 ? (nout + 255) / 256 : 4096);
+        PR_INJECT_LAUNCH();
+        cudaError_t err = reinterpret_cast<AxisLaunch>(e->launch)(a, grid, 256, st);
+        if (err != cudaSuccess) return fail(PR_ERR_CUDA, "axis launch: %s", cudaGetErrorString(err));
+        return PR_OK;
+    }
+    AxisPlan p;
+    pr_status s = axis_plan(a, dtype, op, prec, aux, cfg, &p);
+    if (s != PR_OK) return s;
+    const KernelEntry* e = p.e;
     // the scratch's growth, the two launches and what they leave in it belong
     // together, whatever other host threads enqueue on the stream
     std::unique_lock<std::mutex> pair(g_pair_mu, std::defer_lock);
@@ -832,15 +860,15 @@ static pr_status run_axis(const void* x, int64_t outer, int64_t n, int64_t inner
         if (s != PR_OK) return s;
         a.scratch = sc;
     }
-    const int64_t warps = tiles * a.splits * a.coop;
-    const int wpb = c.block / 32;
+    const int64_t warps = outer * a.groups * a.splits * a.coop;
+    const int wpb = p.block / 32;
     const int64_t grid = (warps + wpb - 1) / wpb;
     if (grid > 0x7fffffff) return fail(PR_ERR_INVALID, "axis reduction too large for one launch");
     PR_INJECT_LAUNCH();
-    cudaError_t err = reinterpret_cast<AxisLaunch>(e->launch)(a, (int)grid, c.block, st);
+    cudaError_t err = reinterpret_cast<AxisLaunch>(e->launch)(a, (int)grid, p.block, st);
     if (err != cudaSuccess) return fail(PR_ERR_CUDA, "axis launch: %s", cudaGetErrorString(err));
     if (a.splits > 1) {
-        const KernelEntry* f = reg_find(KernelKey{K_AXIS_FINISH, (uint8_t)dtype, (uint8_t)op, (uint8_t)prec,
+        const KernelEntry* f = reg_find(KernelKey{K_AXIS_FINISH, (uint8_t)dtype, (uint8_t)op, (uint8_t)p.prec,
                                                   (uint8_t)aux, 0, 0});
         if (!f) return fail(PR_ERR_UNSUPPORTED, "no axis finishing kernel");
         const int64_t per_out = a.splits <= kAxisThreadFinish ? 1 : 32;   // threads per output
@@ -1660,6 +1688,15 @@ pr_status pr_autotune(pr_kind kind, const void* x, int64_t n, const int64_t* off
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     PR_CUDA(cudaStreamIsCapturing(st, &cap));
     if (cap != cudaStreamCaptureStatusNone) return fail(PR_ERR_INVALID, "autotune cannot run during capture");
+    // Calls that take kernels without a configuration keep the one there is:
+    // candidates would differ by noise, or time a kernel that does not run.
+    DevInfo di;
+    if ((s = device_info(&di, nullptr)) != PR_OK) return s;
+    if ((kind == PR_KIND_SEGMENTED && nseg >= kSegGroupMin) ||
+        (kind == PR_KIND_ROWS && rows_by_groups(x, nseg, n / nseg, dtype, di.sms) >= 0)) {
+        if (best) *best = lookup_cfg(kind, dtype, op, precision, kind == PR_KIND_SEGMENTED ? nseg : n);
+        return PR_OK;
+    }
     const int64_t nout = kind == PR_KIND_REDUCE ? 1 : nseg;
     void* dout = nullptr;
     PR_CUDA(cudaMalloc(&dout, (size_t)nout * (8 + sizeof(pr_prod_aux))));
@@ -1699,6 +1736,15 @@ pr_status pr_autotune_axis(const void* x, int64_t outer, int64_t n, int64_t inne
     if (cap != cudaStreamCaptureStatusNone) return fail(PR_ERR_INVALID, "autotune cannot run during capture");
     const int aux = (op == PR_MAX || op == PR_MIN) ? AUX_ARG
                     : (op == PR_PROD && (dtype == PR_F32 || dtype == PR_F64)) ? AUX_PROD : AUX_NONE;
+    // a shape whose splits are shared has its own launch shape (see pr_autotune)
+    const pr_config now = lookup_cfg(PR_KIND_AXIS, dtype, op, precision, outer * n * inner);
+    AxisArgs a{x, outer, n, inner, 0, 1, 0, 1, 1, 0, nullptr, nullptr, nullptr, 0, nullptr};
+    AxisPlan p;
+    if ((s = axis_plan(a, dtype, op, precision, aux, now, &p)) != PR_OK) return s;
+    if (p.shared) {
+        if (best) *best = now;
+        return PR_OK;
+    }
     const int64_t nout = outer * inner;
     void* dout = nullptr;
     PR_CUDA(cudaMalloc(&dout, (size_t)nout * (8 + sizeof(pr_prod_aux))));
