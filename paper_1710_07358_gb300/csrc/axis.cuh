@@ -152,7 +152,9 @@ __global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_
         // split holds fewer than 2^31 rows): three operations an element
         // (pick, compare of bits, select) instead of the accumulator's
         // 64-bit index and its "none yet" test; started at this lane's first
-        // row, then the same steps as add_ordered
+        // row, picked against itself so that a NaN has the bits that later
+        // picks give it (any other payload would read as a change, and take
+        // the index of the next row), then the same steps as add_ordered
         if (has && r0 + ty < r1) {
             float sv[VE];
             int so[VE];
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_
                 axis_load<VB, Ld>(x, slab + r * a.inner, e);
 #pragma unroll
                 for (int k = 0; k < VE; k++) {
-                    sv[k] = e[k];
+                    sv[k] = T::ordered_pick(e[k], e[k]);
                     so[k] = (int)(r - r0);
                 }
             }
