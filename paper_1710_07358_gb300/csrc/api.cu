@@ -605,15 +605,39 @@ static int rows_group_lanes(int64_t rows, int64_t nv, int es, int sms) {
     return gl;
 }
 
+// Long rows that k_rows and k_segmented take although there are enough of them
+// for a block each: forms whose accumulator is light run at the rate of memory
+// in k_rows, whose blocks all end together, while a row a block leaves a last
+// wave of blocks (time by groups over time by k_rows on GB300: fp32 sum [613,
+// 131072] 1.16, [700, 300000] 1.31, [608, 131072] 0.93; bf16 sum of 8192 vectors
+// a row 1.16 at 608 rows and 1.04 at 613, of 5000 vectors 0.85 to 0.99; fp64 sum of
+// 12288 vectors 1.03 to 1.08; the fp64 product, whose group form multiplies on
+// the integer pipes alone, 0.9 at 4096 vectors, 1.07 at 8192, 1.16 at 16384).  With an index
+// or product state k_rows is bound by its own arithmetic and the groups win
+// (fp32 maximum 0.74 to 1.06, product 0.55 to 1.12), but for 32-bit integers
+// when a second wave is nearly empty (1.06 to 1.15 at 613 and 700 rows).  Rows
+// that are not whole vectors would take k_segmented, which is slower still
+// except for very long ones ([613, 300001] 1.21, [613, 131073] 1.06).
+static bool rows_too_long(int64_t rows, int64_t nv, bool whole, int dtype, int op, int aux, int sms) {
+    if (aux == AUX_NONE) {
+        if (!whole) return nv > 16384 && rows < 8 * (int64_t)sms;
+        return nv > (elem_size(dtype) == 2 || (dtype == PR_F64 && op == PR_PROD) ? 6144 : 8192);
+    }
+    return whole && elem_size(dtype) == 4 && !is_float(dtype) && nv > 8192 && rows > 4 * (int64_t)sms &&
+           rows < 5 * (int64_t)sms;
+}
+
 // Lanes per row (log2) of the row kernel by groups, or -1: the call takes the
 // other kernels.
-static int rows_by_groups(const void* x, int64_t rows, int64_t cols, int dtype, int sms) {
+static int rows_by_groups(const void* x, int64_t rows, int64_t cols, int dtype, int op, int aux, int sms) {
     const int es = elem_size(dtype);
     const uintptr_t mis = reinterpret_cast<uintptr_t>(x) % kGroupVec;
     if (rows < 1 || rows > (int64_t)1 << 50 || cols < 1 || mis % es) return -1;
     // whole vectors, or one more where rows start off the vector grid
     const int64_t ve = kGroupVec / es;
-    const int64_t nv = cols % ve == 0 && mis == 0 ? cols / ve : cols / ve + 2;
+    const bool whole = cols % ve == 0 && mis == 0;
+    const int64_t nv = whole ? cols / ve : cols / ve + 2;
+    if (rows_too_long(rows, nv, whole, dtype, op, aux, sms)) return -1;
     return rows_group_lanes(rows, nv, es, sms);
 }
 
@@ -626,7 +650,7 @@ static pr_status run_rows_group(const void* x, int64_t rows, int64_t cols, int d
     DevInfo di;
     pr_status s = device_info(&di, nullptr);
     if (s != PR_OK) return s;
-    const int gl = rows_by_groups(x, rows, cols, dtype, di.sms);
+    const int gl = rows_by_groups(x, rows, cols, dtype, op, aux, di.sms);
     if (gl < 0) return PR_ERR_UNSUPPORTED;
     const int64_t grid = ((rows << gl) + kGroupBlock - 1) / kGroupBlock;
     if (grid > 0x7fffffff) return PR_ERR_UNSUPPORTED;
@@ -1693,7 +1717,7 @@ pr_status pr_autotune(pr_kind kind, const void* x, int64_t n, const int64_t* off
     DevInfo di;
     if ((s = device_info(&di, nullptr)) != PR_OK) return s;
     if ((kind == PR_KIND_SEGMENTED && nseg >= kSegGroupMin) ||
-        (kind == PR_KIND_ROWS && rows_by_groups(x, nseg, n / nseg, dtype, di.sms) >= 0)) {
+        (kind == PR_KIND_ROWS && rows_by_groups(x, nseg, n / nseg, dtype, op, row_aux, di.sms) >= 0)) {
         if (best) *best = lookup_cfg(kind, dtype, op, precision, kind == PR_KIND_SEGMENTED ? nseg : n);
         return PR_OK;
     }
