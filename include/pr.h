@@ -108,12 +108,16 @@ typedef struct {
 /* Kernel families with their own configurations: REDUCE (pr_reduce*),
  * SEGMENTED (pr_segmented_reduce* of fewer than 8192 segments, 512 with argidx
  * or aux, and rows that do not fit ROWS; more segments ignore it), BACKWARD
- * (pr_reduce_backward), ROWS (pr_reduce_rows for few long rows when cols is a
- * whole number of vectors and x is aligned to the vector width; bucketed by
- * rows*cols; shorter or more rows ignore it: groups of lanes take a row each), AXIS
- * (pr_reduce_axis with inner > 1; bucketed by outer*n*inner: block and
- * blocks_per_sm size the warps in flight, unroll the rows in flight per lane,
- * vec_bytes the column vectors when a row is a whole number of them). */
+ * (pr_reduce_backward of rows of more than 32768 elements; shorter rows ignore
+ * it), ROWS (pr_reduce_rows for long rows when cols is a whole number of vectors
+ * and x is aligned to the vector width; bucketed by rows*cols; other rows ignore
+ * it: groups of lanes take a row each), AXIS (pr_reduce_axis with inner > 1;
+ * bucketed by outer*n*inner: block and blocks_per_sm size the warps in flight,
+ * unroll the rows in flight per lane, vec_bytes the column vectors when a row is
+ * a whole number of them.  Where few columns make the rows split, and vec_bytes
+ * is 32, the warps of a block may share a split: block and unroll are then the
+ * library's own).  The autotuner leaves the table alone for calls that ignore
+ * their configuration, and returns the one there is. */
 typedef enum {
     PR_KIND_REDUCE = 0, PR_KIND_SEGMENTED = 1, PR_KIND_BACKWARD = 2, PR_KIND_ROWS = 3, PR_KIND_AXIS = 4
 } pr_kind;

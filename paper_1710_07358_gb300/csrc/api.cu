@@ -749,7 +749,9 @@ static pr_status axis_scratch(cudaStream_t st, size_t bytes, char** out) {
 // the least estimated time.  The input streams in stream_us when the waves of
 // blocks are full (a single wave from 0.9 of the GPU on: with 0.6, which took
 // two splits for three, [64, 577, 768] fp32 maximum with index 33.4 us against
-// 30.7, [3, 10000, 256] fp64 product 36.5 against 22.9); SMs that finish early
+// 30.7, [3, 10000, 256] fp64 product 36.5 against 22.9; it loses on fp64 minimum
+// with index [3, 10000, 256] 24.5 against 27.0, [32, 1024, 768] 59.7 against
+// 61.7); SMs that finish early
 // cost about 0.08 of a wave ([16, 4096, 4096] fp32 sum: 173 us in one wave,
 // 160 in many); a wave about 2 us to start and to combine, a finishing pass as
 // much; the partials `part` of the input's traffic per split.

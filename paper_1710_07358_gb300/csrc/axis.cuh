@@ -115,7 +115,9 @@ __device__ __forceinline__ void axis_load(const typename Ld::In* x, int64_t e0, 
 // COOP: the variant whose blocks' warps share a split (a.coop of them, the
 // whole block).  It is compiled apart because its shared memory and registers
 // cost the other resident warps ([4096, 16, 512] fp64 minimum with index 79 us
-// without it in the kernel, 91 with).
+// without it in the kernel, 91 with).  Its sums spill a little at the compiler's
+// choice of registers (fp32 16 bytes at 64, 16-bit 12 at 80, where the fp64
+// product's state spills 12 too).
 template <class T, int U, int VB, bool COOP>
 __global__ void __launch_bounds__(COOP ? 32 * kAxisCoop : MaxBlock<T>::value) k_axis(AxisArgs a) {
     using Ld = typename T::Ld;

@@ -47,9 +47,10 @@
 //   first kernel takes up to 32 neighbouring segments a warp, through shared
 //   memory where they are short; the second shares the long ones among all
 //   warps, chunk by chunk.  fp32 sum on GB300: 10^6 segments of 24 elements on
-//   average (96 MB) 841 -> 50 us (0.31 of a 6.8 TB/s copy), 65536 of 1000 230
-//   -> 64, 10^5 log-uniform to 16384 316 -> 202, 8192 of 40000 207 -> 207;
-//   maximum with index of the first 976 -> 105, of the last 538 -> 243.  Short
+//   average (96 MB) 840 -> 52 us (0.30 of a 6.8 TB/s copy; launches repeated on
+//   one input, a call through the binding takes 56), 65536 of 1000 231 -> 70,
+//   10^5 log-uniform to 16384 317 -> 212, 8192 of 40000 205 -> 207; maximum with
+//   index of the first 976 -> 105, of the last 538 -> 243.  Short
 //   segments are bound by instructions, about 24 warp instructions a segment
 //   of 24 (ncu: issue slots 60 % busy, no one stall dominant), long ones by HBM.
 //
@@ -1343,8 +1344,9 @@ __device__ __forceinline__ Segs seg_bounds(const int64_t* off, int64_t nseg) {
 // shared memory that the L1 cache needs for the loads in flight of the direct
 // path and of k_seg_long (measured: 8192 segments of 40000 254 us with two
 // stages, 207 with one).  Five blocks an SM: 96 registers, the most that no
-// trait on the fp32 path spills at (10^6 segments of 24: 50 us; six blocks 53,
-// eight 53; 105 against 107 and 118 for the maximum with index).
+// trait of 32-bit types spills at (10^6 segments of 24, summed plainly: 50 us; six
+// blocks 53, eight 53; 105 against 107 and 118 for the maximum with index; the
+// maximum with index of 16-bit types spills 80 bytes).
 constexpr int kSegBlock = 128;
 constexpr int kStageBytes = 4096;    // a warp's stage: one batch
 constexpr int kStageMean = 512;
